@@ -154,16 +154,20 @@ tf_status tf_add_source(tf_handle h, int comp, const int lo[3], const int hi[3],
 tf_status tf_add_probe(tf_handle h, int comp, const int p[3], const double* freqs, int nfreq,
                        int64_t n0, int* id);
 
-/* Advance nsteps >= 0 steps of Algorithm 1 (fused form) on the stream:
- * per step one probe-DFT launch and one fused launch doing the B update with
- * CPML memory, the Js update, the theta-scheme E update with sources, the
- * Mur walls and the non-finite watchdog.  Asynchronous; launch errors are
+/* Advance nsteps >= 0 steps of Algorithm 1 (fused form) on the stream: the B
+ * update with CPML memory, the Js update, the theta-scheme E update with
+ * sources, the Mur walls, the probe DFTs and the non-finite watchdog.  Grids
+ * of up to some 25 million points run in place, a B pass and an E pass per
+ * step; larger ones one fused launch per step or two-step passes
+ * (tf_set_two_step).  The results are the same bits.  Asynchronous; launch errors are
  * returned (the handle is then unusable), device-side errors latch for
  * tf_sync(). */
 tf_status tf_step(tf_handle h, int64_t nsteps);
 
-/* tf_step with per-kernel timing (the library's profiling hook): advances
- * nsteps exactly like tf_step and records a CUDA event pair on the handle's
+/* Steps with per-kernel timing (the profiling hook of the staged kernels: the
+ * fused step and the two-step kernel, which grids that tf_step runs in place
+ * take here as well): advances nsteps to the same bits as tf_step and records
+ * a CUDA event pair on the handle's
  * stream around every kernel it launches.  On return (the stream is
  * synchronised) kernel_ms[k] is the mean duration in ms of one launch of
  * kernel kind k and launches[k] the number of launches, for k = 0 a separate
@@ -188,9 +192,11 @@ tf_status tf_step_timed(tf_handle h, int64_t nsteps, double* kernel_ms, int64_t*
  * single-step kernel moves the rest of the grid twice.  The results are the
  * same bits as single steps.  It is used when the box is not empty, mu is
  * uniform (tf_set_materials) and it is enabled; an odd step count ends with a
- * single step.
- *   tf_set_two_step  planes = 0 disables it for this handle; 4 .. 24 enables
- *                    it with work items of that many planes (24 by default);
+ * single step.  By default tf_step takes it on grids too large to run in
+ * place.
+ *   tf_set_two_step  planes = 0 disables it for this handle; 4 .. 24 asks for
+ *                    it, with work items of that many planes (24 by default),
+ *                    also on grids that would run in place;
  *                    other values TF_EINVAL.  A tuning switch (the project's
  *                    autotuner sets it per grid): results do not change.
  *   tf_two_step_box  the box in storage points, [lo, hi) per axis (all zero
@@ -214,7 +220,9 @@ tf_status tf_set_item_planes(tf_handle h, int planes);
  * and returns, leaving the grid's fields undefined (the context stays
  * usable; reload a checkpoint or rebuild the grid).  polls < 0 restores the
  * default; polls = 0 makes every wait give up at once (a test of the error
- * path).  Applies to the handle's later launches, batched ones included. */
+ * path).  Applies to the handle's later launches, batched ones included; a
+ * handle with a limit of its own takes the staged kernels on grids that would
+ * otherwise run in place. */
 tf_status tf_set_wait_limit(tf_handle h, int64_t polls);
 
 /* Advance n independent grids by nsteps steps each (the batched workload:

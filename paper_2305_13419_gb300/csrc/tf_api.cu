@@ -24,7 +24,8 @@ struct Layout {
     int ncpml_axes;         // axes with a CPML (6 psi arrays each)
     int ntx, nty, nch, kend; // fused-step tiles, z chunks, planes iterated
     size_t off_fields, off_maps, off_psi, off_prof, off_zero, off_probe, off_series, off_scratch,
-        off_tiles, off_order, off_order_s, off_order_t, off_stats, off_coef, off_misc, bytes;
+        off_tiles, off_order, off_order_s, off_order_t, off_stats, off_coef, off_samples, off_misc, bytes;
+    int psa, psb, psc, pnbx, pnby, pnbz;   // items of the steps in place: 2^sa quads x 2^sb rows x 2^sc planes
     long long max_s, max_t;   // capacity of the shell and two-step work lists
     long long scratch_floats;
 };
@@ -59,6 +60,32 @@ tf_status validate(const tf_grid_desc* d) {
     const long long tx = (n[0] + 1 + kSX - 1) / kSX, ty = (n[1] + 1 + kSY - 1) / kSY;
     if (tx * ty > kMaxTiles || n[2] + 1 > kMaxPlanes) return TF_ENOTSUP;
     return TF_OK;
+}
+
+// Shape of the items of the steps in place (a thread has a quad of x points):
+// the fewest threads off the grid; long rows before square ones (with rows of
+// 4 instead of 16 quads a step of the 512 x 256 x 128 CPW took 268 us instead
+// of 251); then few neighbours outside the item along y and z.
+void pass_shape(Layout& L, int cx, int cy) {
+    const int nq = (cx + 3) / 4;
+    double best = 1e300;
+    for (int a = 0; a <= 4; ++a)
+        for (int b = 0; a + b <= kPassBits; ++b) {
+            const int c = kPassBits - a - b;
+            if (c > 0 && (1 << (c - 1)) >= L.kend) continue;
+            const double full = (double)(((nq - 1) >> a) + 1) * (((cy - 1) >> b) + 1) * (((L.kend - 1) >> c) + 1);
+            const double halo = 1.0 + 1.2 / (1 << a) + 0.25 / (1 << b) + 0.25 / (1 << c);
+            const double cost = full * halo;
+            if (cost < best) {
+                best = cost;
+                L.psa = a;
+                L.psb = b;
+                L.psc = c;
+            }
+        }
+    L.pnbx = ((nq - 1) >> L.psa) + 1;
+    L.pnby = ((cy - 1) >> L.psb) + 1;
+    L.pnbz = ((L.kend - 1) >> L.psc) + 1;
 }
 
 Layout layout_of(const tf_grid_desc* d) {
@@ -103,6 +130,8 @@ Layout layout_of(const tf_grid_desc* d) {
     L.max_t = (long long)L.ntx * L.nty * (L.N[2] / kTBLenMin + 1);
     L.off_order_t = o; o += align_up(sizeof(long long) * (size_t)L.max_t);
     L.off_stats = o;  o += align_up(sizeof(StatPartial) * (size_t)(L.N[2] + 1));
+    pass_shape(L, cx, cy);
+    L.off_samples = o; o += align_up(sizeof(float) * kPassSteps * TF_MAX_PROBES);
     L.off_misc = o;   o += kAlign;
     L.bytes = o;
     return L;
@@ -145,7 +174,7 @@ struct tf_ctx {
     int nitems_s, blocks_s, nitems_t, blocks_t;
     unsigned long long* ctr_t;
     unsigned long long base_t;
-    int two_step_on;    // two-step passes allowed (tf_set_two_step; on by default)
+    int two_step_on;    // two-step passes: 0 never, 1 where tf_step's rule takes them (default), 2 asked for
     int item_planes;    // planes per single-step work item (tf_set_item_planes)
     int tb_len;         // planes per two-step work item
     int ppos[TF_MAX_PROBES][3];   // probe points (storage coordinates)
@@ -156,6 +185,7 @@ struct tf_ctx {
     int primed;
     int order_dirty;   // the work-item order must be rebuilt before the next step
     int fine;          // fewer items than CTA slots: every item goes out in pieces
+    int imu_kept;      // the third field buffer's E holds per-face 1/mu (mu varies; no two-step passes then)
     char* ws;
     float* scratch;
     unsigned* status;
@@ -520,6 +550,14 @@ tf_status tf_set_materials(tf_handle h, const float* eps_r, const float* mu_r, c
     TF_CUDA(cudaStreamSynchronize(h->stream));
     TF_CUDA(cudaMemsetAsync(h->status, 0, sizeof(unsigned), h->stream));
     P.uniform_mu = hm[2] ? 0 : 1;
+    if (!P.uniform_mu) {
+        TF_CUDA(launch_face_imu(P, h->fE[2], h->stream));
+        h->imu_kept = 1;
+    } else if (h->imu_kept) {
+        for (int c = 0; c < 3; ++c)
+            TF_CUDA(cudaMemsetAsync(h->fE[2][c], 0, sizeof(float) * (size_t)h->L.total, h->stream));
+        h->imu_kept = 0;
+    }
     if (st & kStatusBadMaterial) return TF_EINVAL;
     float inv_eu, lon;
     memcpy(&inv_eu, &hm[0], 4);
@@ -674,6 +712,61 @@ cudaError_t launch_two_steps(tf_ctx* h, Sources& S, cudaEvent_t* ev) {
     bind(h, h->cur, h->nxt, h->P, h->O);
     h->level += 2;
     return e;
+}
+
+// nsteps steps in place in the current buffer
+cudaError_t run_passes(tf_ctx* h, const Sources& S, int64_t nsteps) {
+    const Layout& L = h->L;
+    PassArgs A;
+    memset(&A, 0, sizeof(A));
+    A.P = h->P;
+    A.S = S;
+    A.tilemat = h->O.tilemat;
+    A.ntx = L.ntx;
+    for (int c = 0; c < 3; ++c) A.imu[c] = h->fE[2][c];
+    A.sa = L.psa;
+    A.sb = L.psb;
+    A.sc = L.psc;
+    A.nbx = L.pnbx;
+    A.nby = L.pnby;
+    A.nbz = L.pnbz;
+    A.cx = h->P.per[0] ? h->P.N[0] : h->P.n[0];
+    A.cy = h->P.per[1] ? h->P.N[1] : h->P.n[1];
+    A.kend = L.kend;
+    A.samples = (float*)(h->ws + L.off_samples);
+    A.nprobe = h->R.n;
+    const int last[3] = {A.cx - 1, A.cy - 1, A.kend - 1};
+    for (int p = 0; p < h->R.n; ++p) {   // the item that samples a probe (a point on a high wall: the item next to it)
+        int w[3];
+        for (int a = 0; a < 3; ++a) w[a] = h->ppos[p][a] < last[a] ? h->ppos[p][a] : last[a];
+        A.pr_block[p] = ((w[2] >> L.psc) * L.pnby + (w[1] >> L.psb)) * L.pnbx + (w[0] >> (L.psa + 2));
+        A.pr_comp[p] = h->R.comp[p];
+        A.pr_q[p] = h->R.q[p];
+    }
+    PassAmps amp[kPassSteps];
+    for (int64_t s = 0; s < nsteps;) {
+        const int m = (int)(nsteps - s < kPassSteps ? nsteps - s : kPassSteps);
+        for (int u = 0; u < m; ++u)
+            for (int q = 0; q < h->nsrc; ++q)
+                amp[u].a[q] = (float)(h->src[q].amp * waveform(h->src[q], (double)(h->level + u + 1) * h->dt));
+        const cudaError_t e = launch_passes(A, h->R, amp, h->level, m, h->stream);
+        if (e != cudaSuccess) return e;
+        h->level += m;
+        s += m;
+    }
+    return cudaSuccess;
+}
+
+// Does tf_step run in place (tf_pass.cu)?  Not when two-step passes were
+// asked for, nor under a wait limit of the handle's own (the passes wait for
+// nothing).  us per step in place / single staged steps / two-step passes on
+// CPW grids: 0.3 M cells 7 / 21 / 68, 2.1 M 43 / 72 / 126, 4 M 72 / 104 / 149,
+// 8 M 132 / 165 / 182, 17 M 251 / 266 / 273, 25 M 373 / 384 / 369, 43 M 640 /
+// 627 / 600: once E and B have left the L2 cache the 72 bytes per point of the
+// two passes cost more than the staged kernels' 48 and 24.
+bool in_place(const tf_ctx* h) {
+    const bool asked = h->two_step_on == 2 && h->box_ok && h->P.uniform_mu;
+    return !asked && h->P.wait_polls == kSpinLimit && h->L.total <= kPassPoints;
 }
 
 bool two_step(const tf_ctx* h) { return h->two_step_on && h->box_ok && h->P.uniform_mu && h->nitems_t > 0; }
@@ -836,6 +929,10 @@ tf_status tf_step(tf_handle h, int64_t nsteps) {
     }
     Sources S;
     fill_sources(h, S);
+    if (in_place(h)) {
+        TF_CUDA(run_passes(h, S, nsteps));
+        return TF_OK;
+    }
     TF_CUDA(refresh_order(h, S));
     int64_t s = 0;
     if (two_step(h))
@@ -846,7 +943,7 @@ tf_status tf_step(tf_handle h, int64_t nsteps) {
 
 tf_status tf_set_two_step(tf_handle h, int planes) {
     if (!h || (planes != 0 && (planes < kTBLenMin || planes > kTBLenMax))) return TF_EINVAL;
-    h->two_step_on = planes != 0;
+    h->two_step_on = planes != 0 ? 2 : 0;
     if (planes != 0 && planes != h->tb_len) {
         h->tb_len = planes;
         h->order_dirty = 1;   // the box's work list is cut again
@@ -877,7 +974,7 @@ tf_status tf_two_step_box(tf_handle h, int lo[3], int hi[3], int* active) {
     hi[1] = h->ty1 * kSY;
     lo[2] = h->tz0;
     hi[2] = h->tz1;
-    if (active) *active = two_step(h) ? 1 : 0;
+    if (active) *active = two_step(h) && !in_place(h) ? 1 : 0;
     return TF_OK;
 }
 
@@ -1266,7 +1363,8 @@ int ckpt_parts(const tf_ctx* h, CkptPart* parts) {
     const size_t fb = sizeof(float) * (size_t)h->L.total;
     const int x = h->cur, y = h->nxt, z = 3 - h->cur - h->nxt;
     int n = 0;
-    for (int c = 0; c < 3; ++c) parts[n++] = {h->fE[x][c], {h->fE[y][c], h->fE[z][c]}, fb};
+    // (where mu varies the third buffer's E holds 1/mu: there are no two-step passes then)
+    for (int c = 0; c < 3; ++c) parts[n++] = {h->fE[x][c], {h->fE[y][c], h->imu_kept ? nullptr : h->fE[z][c]}, fb};
     for (int c = 0; c < 3; ++c) parts[n++] = {h->fB[x][c], {h->fB[y][c], h->fB[z][c]}, fb};
     for (int c = 0; c < 3; ++c) parts[n++] = {h->fJ[x][c], {h->fJ[y][c], h->fJ[z][c]}, fb};
     for (int a = 0; a < 3; ++a) {

@@ -341,6 +341,32 @@ __host__ __device__ __forceinline__ long long item_with_grid(long long d, int gr
 cudaError_t launch_step_batch(const BatchLaunch& BL, int blocks, cudaStream_t st);
 cudaError_t launch_step_advance(int* step, cudaStream_t st);
 
+// Steps in place by a B pass and an E pass each (tf_pass.cu): the fields are
+// those of the current buffer.
+constexpr int kPassSteps = 32;     // steps per group of launches (probe samples are kept for that many)
+constexpr long long kPassPoints = 24LL << 20;   // padded points of a grid up to which tf_step runs in place
+constexpr int kPassBits = 7, kPassThreads = 1 << kPassBits;   // threads of an item, a quad of x points each
+struct PassArgs {
+    Params P;
+    Sources S;                                  // amplitudes come from PassAmps
+    const float4* tilemat;                      // tile-plane records of the single-step kernel
+    int ntx;
+    const float* imu[3];                        // per-face 1/mu where mu varies
+    int sa, sb, sc;                             // an item: 2^sa quads x 2^sb rows x 2^sc planes
+    int nbx, nby, nbz;                          // items along x, y, z
+    int cx, cy, kend;                           // points advanced along x, y, z: [0, c)
+    int nprobe;
+    int pr_block[TF_MAX_PROBES], pr_comp[TF_MAX_PROBES];   // the item that samples a probe
+    long long pr_q[TF_MAX_PROBES];
+    float* samples;                             // [step][probe]: E^n of the steps
+};
+struct PassAmps {
+    float a[TF_MAX_SOURCES];                    // amp * s(t^{n+1}) of a step
+};
+cudaError_t launch_passes(const PassArgs& A, const Probes& R, const PassAmps* amp, long long level, int steps,
+                          cudaStream_t st);
+cudaError_t launch_face_imu(const Params& P, float* const w[3], cudaStream_t st);
+
 // launchers (tf_kernels.cu)
 cudaError_t launch_convert_materials(const Params& P, const float* eps_r, const float* mu_r,
                                      const float* lam, const float* sigma, double dt,

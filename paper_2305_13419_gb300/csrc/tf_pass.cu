@@ -1,0 +1,593 @@
+// tf_pass.cu -- the fused leapfrog in place, two passes per step (sm_103a).
+//
+// Algorithm 1 (arXiv 2305.13419, Sec. 3) in its fused leapfrog form is
+//   B pass  Bt^{n+1/2} = Bt^{n-1/2} - curl(E^n)                    (CPML psi_B)
+//   E pass  Jt^{n+1/2} = Jt^{n-1/2} + kt_e E^n,
+//           E^{n+1}    = ca E^n + cb (curl(Bt/mu) - Jt^{n+1/2})      (CPML psi_E)
+// each of which may run in place: the B pass reads its neighbours' E and only
+// its own B, the E pass its neighbours' B and only its own E.
+//
+// A thread owns four x-adjacent points (128-bit accesses); its arithmetic is
+// the packed FP32x2 add / sub / mul / fma of the single-step kernel in the
+// same order, so the two give the same bits.  There is no staging, no barrier
+// and no ring to fill: a pass is a launch of independent threads, each with
+// one round of loads in flight.  That moves 72 bytes per point and step where
+// the staged kernel moves 48, but in place (24 bytes of E and B per point
+// where that one keeps two buffers), so that up to a few million points it
+// all stays in the L2 cache, and a small grid is not held up by a chain of
+// planes per CTA.
+#include <math.h>
+
+#include "tf_device.cuh"
+#include "tf_internal.cuh"
+
+namespace tf {
+
+namespace {
+
+using namespace dev;
+
+constexpr int kFT = kPassThreads;
+constexpr int kFMin = 5;   // resident CTAs per SM: 20 warps of 96 registers
+
+// four x-adjacent values: lanes 0, 1 in v[0], lanes 2, 3 in v[1]
+struct Q4 {
+    f2 v[2];
+};
+__device__ __forceinline__ Q4 ld4(const float* p) {
+    const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(p);
+    return {{t.x, t.y}};
+}
+__device__ __forceinline__ void st4(float* p, const Q4& q) {
+    *reinterpret_cast<ulonglong2*>(p) = make_ulonglong2(q.v[0], q.v[1]);
+}
+// lanes whose bit is set in m take nv, the others ov
+__device__ __forceinline__ Q4 sel4(const Q4& nv, const Q4& ov, unsigned m) {
+    return {{sel2(nv.v[0], ov.v[0], m & 3u), sel2(nv.v[1], ov.v[1], m >> 2)}};
+}
+// products rounded on their own
+__device__ __forceinline__ Q4 rnd4(const Q4& a, const Q4& b) {
+    return {{pk(__fmul_rn(lo(a.v[0]), lo(b.v[0])), __fmul_rn(hi(a.v[0]), hi(b.v[0]))),
+             pk(__fmul_rn(lo(a.v[1]), lo(b.v[1])), __fmul_rn(hi(a.v[1]), hi(b.v[1])))}};
+}
+// store the lanes of m over the old values (the whole quad is this thread's)
+__device__ __forceinline__ void st4m(float* p, const Q4& nv, const Q4& ov, unsigned m) {
+    if (m == 15u)
+        st4(p, nv);
+    else if (m)
+        st4(p, sel4(nv, ov, m));
+}
+// lanes shifted by one: the next higher / lower x neighbour of each lane
+__device__ __forceinline__ Q4 up4(const Q4& q, float next) {
+    return {{pk(hi(q.v[0]), lo(q.v[1])), pk(hi(q.v[1]), next)}};
+}
+__device__ __forceinline__ Q4 dn4(const Q4& q, float prev) {
+    return {{pk(prev, lo(q.v[0])), pk(hi(q.v[0]), lo(q.v[1]))}};
+}
+__device__ __forceinline__ float lane(const Q4& q, int p) {
+    const f2 v = p < 2 ? q.v[0] : q.v[1];
+    return p & 1 ? hi(v) : lo(v);
+}
+__device__ __forceinline__ Q4 set_lane(const Q4& q, int p, float x) {
+    Q4 r = q;
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+        if (u == p) r.v[u >> 1] = u & 1 ? pk(lo(r.v[u >> 1]), x) : pk(x, hi(r.v[u >> 1]));
+    return r;
+}
+__device__ __forceinline__ Q4 sub4(const Q4& a, const Q4& b) { return {{sub2(a.v[0], b.v[0]), sub2(a.v[1], b.v[1])}}; }
+__device__ __forceinline__ Q4 add4(const Q4& a, const Q4& b) { return {{add2(a.v[0], b.v[0]), add2(a.v[1], b.v[1])}}; }
+__device__ __forceinline__ Q4 mul4(const Q4& a, const Q4& b) { return {{mul2(a.v[0], b.v[0]), mul2(a.v[1], b.v[1])}}; }
+__device__ __forceinline__ Q4 fma4(const Q4& a, const Q4& b, const Q4& c) {
+    return {{fma2(a.v[0], b.v[0], c.v[0]), fma2(a.v[1], b.v[1], c.v[1])}};
+}
+__device__ __forceinline__ Q4 neg4(const Q4& a) {
+    const f2 s = 0x8000000080000000ull;
+    return {{a.v[0] ^ s, a.v[1] ^ s}};
+}
+__device__ __forceinline__ Q4 all4(float x) {
+    const f2 v = pk(x, x);
+    return {{v, v}};
+}
+
+// the quad of a thread: its points and the lanes each component advances
+struct Quad {
+    int x, j, k;
+    unsigned o;          // byte offset in a field array
+    unsigned hv, in;     // lanes with a half / an integer position off the walls along x
+    unsigned sx;         // lanes inside the CPML slabs of the x axis
+    bool iny, inz;       // the row / plane is off the low walls
+    bool sy, sz;         // the row / plane is inside a CPML slab
+    bool full;           // every lane of every component advances
+};
+__device__ __forceinline__ Quad quad_of(const Params& P, int x, int j, int k) {
+    Quad u;
+    u.x = x;
+    u.j = j;
+    u.k = k;
+    u.o = 4u * (unsigned)(k * (int)P.plane + j * P.pitch + x);
+    const int hx = P.per[0] ? P.N[0] : P.n[0];   // points advanced along x: [lo, hx)
+    u.hv = x + 4 <= hx ? 15u : x < hx ? (1u << (hx - x)) - 1u : 0u;
+    u.in = (!P.per[0] && x == 0) ? u.hv & 14u : u.hv;
+    u.sx = 0u;
+    const int L = P.L[0];
+    if (L > 0 && (x < L || x + 3 >= P.n[0] - L)) {
+#pragma unroll
+        for (int p = 0; p < 4; ++p) u.sx |= (x + p < L || x + p >= P.n[0] - L) ? 1u << p : 0u;
+        u.sx &= u.hv;
+    }
+    u.iny = P.per[1] || j >= 1;
+    u.inz = P.per[2] || k >= 1;
+    u.sy = in_slab(P, 1, j);
+    u.sz = in_slab(P, 2, k);
+    u.full = u.in == 15u && u.iny && u.inz;
+    return u;
+}
+
+// soft sources of step t at a quad
+__device__ __forceinline__ void add_src(const Sources& S, const PassAmps& W, int x, int j, int k, Q4& nx, Q4& ny, Q4& nz) {
+    Q4 ax = {{0, 0}}, ay = ax, az = ax;
+    for (int s = 0; s < S.n; ++s) {
+        if (j < S.lo[s][1] || j >= S.hi[s][1] || k < S.lo[s][2] || k >= S.hi[s][2]) continue;
+        const float v = W.a[s];
+        const int x0 = S.lo[s][0], x1 = S.hi[s][0];
+        const Q4 a = {{pk(x >= x0 && x < x1 ? v : 0.f, x + 1 >= x0 && x + 1 < x1 ? v : 0.f),
+                       pk(x + 2 >= x0 && x + 2 < x1 ? v : 0.f, x + 3 >= x0 && x + 3 < x1 ? v : 0.f)}};
+        if (S.comp[s] == 0)
+            ax = add4(ax, a);
+        else if (S.comp[s] == 1)
+            ay = add4(ay, a);
+        else
+            az = add4(az, a);
+    }
+    nx = add4(nx, ax);
+    ny = add4(ny, ay);
+    nz = add4(nz, az);
+}
+
+// own values that a pass needs and that nobody else writes: read past L1, so
+// that they may be fetched while the pass before is still running elsewhere
+__device__ __forceinline__ Q4 own4(const float* base, unsigned o) {
+    Q4 q;
+    asm volatile("ld.global.cg.v2.u64 {%0, %1}, [%2];" : "=l"(q.v[0]), "=l"(q.v[1]) : "l"((const char*)base + o) : "memory");
+    return q;
+}
+// accesses at a 32-bit byte offset from a uniform base
+__device__ __forceinline__ Q4 ldo(const float* base, unsigned o) { return ld4((const float*)((const char*)base + o)); }
+__device__ __forceinline__ void sto(float* base, unsigned o, const Q4& q) { st4((float*)((char*)base + o), q); }
+__device__ __forceinline__ float ldf(const float* base, unsigned o) { return *(const float*)((const char*)base + o); }
+
+// profile of the x axis at a quad, zero off its slab lanes
+__device__ __forceinline__ Q4 prof_x(const float* pf, const Quad& u) {
+    const Q4 z = {{0, 0}};
+    return sel4(ld4(pf + u.x), z, u.sx);
+}
+
+struct PreB {
+    Q4 ox, oy, oz;       // B
+    Q4 z0, z1, x0, x1, y0, y1;   // psi_B pairs of the slab axes z, x, y
+    float bz, cz, by, cy;        // CPML coefficients of the plane and the row
+};
+template <bool kPlain>
+__device__ __forceinline__ void pre_b(const Params& P, const Quad& u, PreB& r) {
+    r.ox = own4(P.B[0], u.o);
+    r.oy = own4(P.B[1], u.o);
+    r.oz = own4(P.B[2], u.o);
+    if (kPlain) return;
+    if (u.sz) {
+        r.z0 = own4(P.psiB[0][2], u.o);
+        r.z1 = own4(P.psiB[1][2], u.o);
+        r.bz = __ldg(P.pbB[2] + u.k);
+        r.cz = __ldg(P.pcB[2] + u.k);
+    }
+    if (u.sx) {
+        r.x0 = own4(P.psiB[1][0], u.o);
+        r.x1 = own4(P.psiB[2][0], u.o);
+    }
+    if (u.sy) {
+        r.y0 = own4(P.psiB[0][1], u.o);
+        r.y1 = own4(P.psiB[2][1], u.o);
+        r.by = __ldg(P.pbB[1] + u.j);
+        r.cy = __ldg(P.pcB[1] + u.j);
+    }
+}
+// CPML memory pair: n = b psi + c d, stored on the lanes of m
+__device__ __forceinline__ void psi_new(float* w1, float* w2, unsigned o, const Q4& b, const Q4& c, const Q4& o1,
+                                        const Q4& o2, const Q4& d1, const Q4& d2, unsigned m1, unsigned m2, Q4& n1,
+                                        Q4& n2) {
+    n1 = fma4(b, o1, mul4(c, d1));
+    n2 = fma4(b, o2, mul4(c, d2));
+    st4m((float*)((char*)w1 + o), n1, o1, m1);
+    st4m((float*)((char*)w2 + o), n2, o2, m2);
+}
+
+template <bool kPlain>
+__device__ __forceinline__ void post_b(const Params& P, const Quad& u, const PreB& r) {
+    const unsigned o = u.o, row = 4u * (unsigned)P.pitch, pl = 4u * (unsigned)P.plane;
+    unsigned oy1 = o + row, oz1 = o + pl, on = o + 16u;
+    bool wrap = false;
+    if (!kPlain) {
+        if (u.j + 1 == P.N[1]) oy1 = o - (unsigned)u.j * row;
+        if (u.k + 1 == P.N[2]) oz1 = o - (unsigned)u.k * pl;
+        // the point past the quad; at the row's end the wrap to x = 0 (on a walled axis: nothing keeps it)
+        if (u.x + 4 >= P.N[0]) on = o - 4u * (unsigned)u.x;
+        wrap = P.per[0] && u.x + 4 > P.N[0];
+    }
+    const Q4 ex = ldo(P.E[0], o), ey = ldo(P.E[1], o), ez = ldo(P.E[2], o);
+    const Q4 ex_y = ldo(P.E[0], oy1), ez_y = ldo(P.E[2], oy1);
+    const Q4 ex_z = ldo(P.E[0], oz1), ey_z = ldo(P.E[1], oz1);
+    const float ey_n = ldf(P.E[1], on), ez_n = ldf(P.E[2], on);
+    Q4 ey_x = up4(ey, ey_n), ez_x = up4(ez, ez_n);
+    if (!kPlain && wrap) {   // the row ends inside the quad: its last point wraps
+        ey_x = set_lane(ey_x, P.N[0] - 1 - u.x, ey_n);
+        ez_x = set_lane(ez_x, P.N[0] - 1 - u.x, ez_n);
+    }
+    const Q4 r0 = all4(P.r[0]), r1 = all4(P.r[1]), r2 = all4(P.r[2]);
+    const Q4 dEz_y = sub4(ez_y, ez), dEx_y = sub4(ex_y, ex), dEy_z = sub4(ey_z, ey), dEx_z = sub4(ex_z, ex);
+    const Q4 dEz_x = sub4(ez_x, ez), dEy_x = sub4(ey_x, ey);
+    Q4 bx = fma4(r2, dEy_z, sub4(r.ox, mul4(r1, dEz_y)));
+    Q4 by = fma4(r0, dEz_x, sub4(r.oy, mul4(r2, dEx_z)));
+    Q4 bz = fma4(r1, dEx_y, sub4(r.oz, mul4(r0, dEy_x)));
+    if (!kPlain) {
+        const unsigned mx = u.in, my = u.iny ? u.hv : 0u, mz = u.inz ? u.hv : 0u;
+        Q4 n1, n2;
+        if (u.sz) {
+            psi_new(P.psiB[0][2], P.psiB[1][2], o, all4(r.bz), all4(r.cz), r.z0, r.z1,
+                    dEy_z, dEx_z, mx, my, n1, n2);
+            bx = add4(bx, n1);
+            by = sub4(by, n2);
+        }
+        if (u.sx) {
+            psi_new(P.psiB[1][0], P.psiB[2][0], o, prof_x(P.pbB[0], u), prof_x(P.pcB[0], u), r.x0, r.x1, dEz_x, dEy_x,
+                    u.sx & my, u.sx & mz, n1, n2);
+            by = add4(by, n1);
+            bz = sub4(bz, n2);
+        }
+        if (u.sy) {
+            psi_new(P.psiB[0][1], P.psiB[2][1], o, all4(r.by), all4(r.cy), r.y0, r.y1,
+                    dEz_y, dEx_y, mx, mz, n1, n2);
+            bx = sub4(bx, n1);
+            bz = add4(bz, n2);
+        }
+        if (!u.full) {
+            bx = sel4(bx, r.ox, mx);
+            by = sel4(by, r.oy, my);
+            bz = sel4(bz, r.oz, mz);
+        }
+    }
+    sto(P.B[0], o, bx);
+    sto(P.B[1], o, by);
+    sto(P.B[2], o, bz);
+}
+
+struct PreE {
+    Q4 ex, ey, ez;               // E
+    Q4 z0, z1, x0, x1, y0, y1;   // psi_E pairs of the slab axes z, x, y
+    float bz, cz, by, cy;        // CPML coefficients of the plane and the row
+    float4 rec;
+};
+template <bool kPlain>
+__device__ __forceinline__ void pre_e(const PassArgs& A, const Quad& u, PreE& r) {
+    const Params& P = A.P;
+    r.rec = __ldg(A.tilemat + (long long)((u.j / kSY) * A.ntx + u.x / kSX) * P.N[2] + u.k);
+    r.ex = own4(P.E[0], u.o);
+    r.ey = own4(P.E[1], u.o);
+    r.ez = own4(P.E[2], u.o);
+    if (!kPlain) {
+        if (u.sz) {
+            r.z0 = own4(P.psiE[0][2], u.o);
+            r.z1 = own4(P.psiE[1][2], u.o);
+            r.bz = __ldg(P.pbE[2] + u.k);
+            r.cz = __ldg(P.pcE[2] + u.k);
+        }
+        if (u.sx) {
+            r.x0 = own4(P.psiE[1][0], u.o);
+            r.x1 = own4(P.psiE[2][0], u.o);
+        }
+        if (u.sy) {
+            r.y0 = own4(P.psiE[0][1], u.o);
+            r.y1 = own4(P.psiE[2][1], u.o);
+            r.by = __ldg(P.pbE[1] + u.j);
+            r.cy = __ldg(P.pcE[1] + u.j);
+        }
+    }
+}
+
+template <bool kPlain>
+__device__ __forceinline__ void post_e(const PassArgs& A, const Quad& u, const PreE& r, const PassAmps& W) {
+    const Params& P = A.P;
+    const unsigned o = u.o, row = 4u * (unsigned)P.pitch, pl = 4u * (unsigned)P.plane;
+    unsigned oy1 = o - row, oz1 = o - pl, op = o - 4u;
+    if (!kPlain) {   // below a low wall: the own value, whose difference nothing keeps
+        if (u.j == 0) oy1 = P.per[1] ? o + (unsigned)(P.N[1] - 1) * row : o;
+        if (u.k == 0) oz1 = P.per[2] ? o + (unsigned)(P.N[2] - 1) * pl : o;
+        if (u.x == 0) op = P.per[0] ? o + 4u * (unsigned)(P.N[0] - 1) : o;
+    }
+    const Q4 hx = ldo(P.B[0], o), hy = ldo(P.B[1], o), hz = ldo(P.B[2], o);
+    const Q4 hx_zm = ldo(P.B[0], oz1), hy_zm = ldo(P.B[1], oz1);
+    const Q4 hx_ym = ldo(P.B[0], oy1), hz_ym = ldo(P.B[2], oy1);
+    const float hy_p = ldf(P.B[1], op), hz_p = ldf(P.B[2], op);
+    // (the first use of the record: every load above is on its way by now)
+    const bool coef = isnan(r.rec.x), sc = coef || r.rec.z > 0.f;   // per-point coefficients; Js advances on the tile-plane
+    Q4 ojx, ojy, ojz;
+    if (sc) {
+        ojx = ldo(P.J[0], o);
+        ojy = ldo(P.J[1], o);
+        ojz = ldo(P.J[2], o);
+    }
+    Q4 dHz_y, dHy_z, dHx_z, dHz_x, dHy_x, dHx_y;
+    if (kPlain || P.uniform_mu) {
+        dHz_y = sub4(hz, hz_ym);
+        dHy_z = sub4(hy, hy_zm);
+        dHx_z = sub4(hx, hx_zm);
+        dHz_x = sub4(hz, dn4(hz, hz_p));
+        dHy_x = sub4(hy, dn4(hy, hy_p));
+        dHx_y = sub4(hx, hx_ym);
+    } else {
+        // differences of H = B / mu, rounded as the single-step kernel's: both
+        // products on their own (rnd4: no product may move into a fused
+        // multiply-add), but for dHx_y where the tile-plane's material varies
+        const Q4 wx = ldo(A.imu[0], o), wy = ldo(A.imu[1], o), wz = ldo(A.imu[2], o);
+        auto diff = [&](const Q4& h, const Q4& w, const Q4& hm, const Q4& wm) { return sub4(rnd4(h, w), rnd4(hm, wm)); };
+        dHz_y = diff(hz, wz, hz_ym, ldo(A.imu[2], oy1));
+        const Q4 wx_y = ldo(A.imu[0], oy1);
+        dHx_y = coef ? fma4(neg4(hx_ym), wx_y, rnd4(hx, wx)) : diff(hx, wx, hx_ym, wx_y);
+        dHy_z = diff(hy, wy, hy_zm, ldo(A.imu[1], oz1));
+        dHx_z = diff(hx, wx, hx_zm, ldo(A.imu[0], oz1));
+        dHz_x = diff(hz, wz, dn4(hz, hz_p), dn4(wz, ldf(A.imu[2], op)));
+        dHy_x = diff(hy, wy, dn4(hy, hy_p), dn4(wy, ldf(A.imu[1], op)));
+    }
+    const Q4 r0 = all4(P.r[0]), r1 = all4(P.r[1]), r2 = all4(P.r[2]);
+    Q4 cx = sub4(mul4(r1, dHz_y), mul4(r2, dHy_z));
+    Q4 cy = sub4(mul4(r2, dHx_z), mul4(r0, dHz_x));
+    Q4 cz = sub4(mul4(r0, dHy_x), mul4(r1, dHx_y));
+    const unsigned mx = kPlain ? 15u : u.iny && u.inz ? u.hv : 0u, my = kPlain ? 15u : u.inz ? u.in : 0u,
+                   mz = kPlain ? 15u : u.iny ? u.in : 0u;
+    if (!kPlain) {
+        Q4 n1, n2;
+        if (u.sz) {
+            psi_new(P.psiE[0][2], P.psiE[1][2], o, all4(r.bz), all4(r.cz), r.z0, r.z1,
+                    dHy_z, dHx_z, mx, my, n1, n2);
+            cx = sub4(cx, n1);
+            cy = add4(cy, n2);
+        }
+        if (u.sx) {
+            psi_new(P.psiE[1][0], P.psiE[2][0], o, prof_x(P.pbE[0], u), prof_x(P.pcE[0], u), r.x0, r.x1, dHz_x, dHy_x,
+                    u.sx & my, u.sx & mz, n1, n2);
+            cy = sub4(cy, n1);
+            cz = add4(cz, n2);
+        }
+        if (u.sy) {
+            psi_new(P.psiE[0][1], P.psiE[2][1], o, all4(r.by), all4(r.cy), r.y0, r.y1,
+                    dHz_y, dHx_y, mx, mz, n1, n2);
+            cx = add4(cx, n1);
+            cz = sub4(cz, n2);
+        }
+    }
+    if (sc) {
+        Q4 jx, jy, jz;
+        if (coef) {
+            jx = fma4(ldo(P.cj[0], o), r.ex, ojx);
+            jy = fma4(ldo(P.cj[1], o), r.ey, ojy);
+            jz = fma4(ldo(P.cj[2], o), r.ez, ojz);
+        } else {
+            const Q4 cj = all4(r.rec.z);
+            jx = fma4(cj, r.ex, ojx);
+            jy = fma4(cj, r.ey, ojy);
+            jz = fma4(cj, r.ez, ojz);
+        }
+        cx = sub4(cx, jx);
+        cy = sub4(cy, jy);
+        cz = sub4(cz, jz);
+        st4m((float*)((char*)P.J[0] + o), jx, ojx, mx);
+        st4m((float*)((char*)P.J[1] + o), jy, ojy, my);
+        st4m((float*)((char*)P.J[2] + o), jz, ojz, mz);
+    }
+    Q4 nx, ny, nz;
+    if (coef) {
+        nx = fma4(ldo(P.cb[0], o), cx, mul4(ldo(P.ca[0], o), r.ex));
+        ny = fma4(ldo(P.cb[1], o), cy, mul4(ldo(P.ca[1], o), r.ey));
+        nz = fma4(ldo(P.cb[2], o), cz, mul4(ldo(P.ca[2], o), r.ez));
+    } else {
+        const Q4 ca = all4(r.rec.x), cb = all4(r.rec.y);
+        nx = fma4(cb, cx, mul4(ca, r.ex));
+        ny = fma4(cb, cy, mul4(ca, r.ey));
+        nz = fma4(cb, cz, mul4(ca, r.ez));
+    }
+    const Sources& S = A.S;
+    if (S.n > 0 && u.x + 3 >= S.bb_lo[0] && u.x < S.bb_hi[0] && u.j >= S.bb_lo[1] && u.j < S.bb_hi[1] &&
+        u.k >= S.bb_lo[2] && u.k < S.bb_hi[2])
+        add_src(S, W, u.x, u.j, u.k, nx, ny, nz);
+    if (kPlain || u.full) {
+        sto(P.E[0], o, nx);
+        sto(P.E[1], o, ny);
+        sto(P.E[2], o, nz);
+    } else {   // (a component held on a low z wall plane is not stored: a Mur update of that wall is another thread's)
+        nx = sel4(nx, r.ex, mx);
+        ny = sel4(ny, r.ey, my);
+        nz = sel4(nz, r.ez, mz);
+        if (mx) sto(P.E[0], o, nx);
+        if (my) sto(P.E[1], o, ny);
+        if (mz) sto(P.E[2], o, nz);
+    }
+    const Q4 sum = add4(add4(nx, ny), nz);
+    if (!isfinite(lo(sum.v[0]) + hi(sum.v[0])) || !isfinite(lo(sum.v[1]) + hi(sum.v[1])))
+        atomicOr(P.status, kStatusNonFinite);
+    // first-order Mur on the z walls: E_w^{n+1} = E_i^n + M (E_i^{n+1} - E_w^n)
+    if (!kPlain && P.bc[2] == TF_BC_MUR && (u.k == 1 || u.k == P.n[2] - 1)) {
+        const unsigned wx = u.iny ? u.hv : 0u, wy = u.in;
+#pragma unroll
+        for (int w = 0; w < 2; ++w) {
+            if (u.k != (w ? P.n[2] - 1 : 1)) continue;
+            const unsigned ow = w ? o + pl : o - pl;
+#pragma unroll
+            for (int p = 0; p < 4; ++p) {
+                float* e0 = (float*)((char*)P.E[0] + ow) + p;
+                float* e1 = (float*)((char*)P.E[1] + ow) + p;
+                if (wx >> p & 1u) *e0 = lane(r.ex, p) + P.mur_M * (lane(nx, p) - *e0);
+                if (wy >> p & 1u) *e1 = lane(r.ey, p) + P.mur_M * (lane(ny, p) - *e1);
+            }
+        }
+    }
+}
+
+// does an item of points [x0, x1) x [y0, y1) x [z0, z1) stay off the walls, the seams and the CPML slabs?
+__device__ __forceinline__ bool plain_item(const Params& P, int x0, int x1, int y0, int y1, int z0, int z1) {
+    const int a0[3] = {x0, y0, z0}, a1[3] = {x1, y1, z1};
+    bool ok = P.uniform_mu && P.bc[2] != TF_BC_MUR;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const int lo_ = P.L[a] > 1 ? P.L[a] : 1, hi_ = P.per[a] ? P.N[a] - 1 : P.n[a] - P.L[a];
+        ok = ok && a0[a] >= lo_ && a1[a] <= hi_;
+    }
+    return ok;
+}
+
+struct Item {
+    bool live, plain;
+    Quad u;
+};
+__device__ __forceinline__ Item item_at(const PassArgs& A, int bx, int by, int bz) {
+    Item it;
+    const int tid = threadIdx.x;
+    const int iq = tid & ((1 << A.sa) - 1), jr = (tid >> A.sa) & ((1 << A.sb) - 1), kr = tid >> (A.sa + A.sb);
+    const int x0 = 4 * (bx << A.sa), y0 = by << A.sb, z0 = bz << A.sc;
+    const int x = x0 + 4 * iq, j = y0 + jr, k = z0 + kr;
+    it.live = x < A.cx && j < A.cy && k < A.kend;
+    it.plain = plain_item(A.P, x0, x0 + (4 << A.sa), y0, y0 + (1 << A.sb), z0, z0 + (1 << A.sc));
+    it.u = quad_of(A.P, x, j, k);
+    return it;
+}
+__device__ __forceinline__ void sample(const PassArgs& A, int blk, int t) {
+    if (threadIdx.x < A.nprobe && A.pr_block[threadIdx.x] == blk)
+        A.samples[t * TF_MAX_PROBES + threadIdx.x] = A.P.E[A.pr_comp[threadIdx.x]][A.pr_q[threadIdx.x]];
+}
+
+}  // namespace
+
+// One pass of one step over the grid (kE: the E pass).  Bound by the latency
+// of its one round of loads on small grids and by memory on large ones: a step
+// of the 512 x 256 x 128 CPW takes 251 us (5.8 TB/s of the 72 bytes per point
+// plus the CPML memories), of the 256 x 128 x 64 CPW 43 us, of a 1 x 1 x 4480
+// column 7 us (two launches).  Quads and 96 registers (20 warps per SM) beat
+// 64 registers and 32 warps (spills: 54 against 52 us on the 256 x 128 x 64
+// CPW); columns of 4 planes per thread took 55 there.
+// Launches overlap (programmatic dependent launch): a thread fetches what
+// only its own pass writes -- one step and two launches ago -- before it waits
+// for the launch before.  That launch lets the next one start only once its
+// own wait is over, so the launch before it is complete by then.
+template <bool kE>
+__global__ void __launch_bounds__(kFT, kFMin) k_pass(const __grid_constant__ PassArgs A, const __grid_constant__ PassAmps W, int t) {
+    const Item it = item_at(A, blockIdx.x, blockIdx.y, blockIdx.z);
+    if (kE) {
+        PreE r;
+        if (it.plain) {
+            pre_e<true>(A, it.u, r);
+            asm volatile("griddepcontrol.wait;" ::: "memory");
+            asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+            post_e<true>(A, it.u, r, W);
+        } else {
+            if (it.live) pre_e<false>(A, it.u, r);
+            asm volatile("griddepcontrol.wait;" ::: "memory");
+            asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+            if (it.live) post_e<false>(A, it.u, r, W);
+        }
+    } else {
+        PreB r;
+        if (it.plain) {
+            pre_b<true>(A.P, it.u, r);
+            asm volatile("griddepcontrol.wait;" ::: "memory");
+            asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+            post_b<true>(A.P, it.u, r);
+        } else {
+            if (it.live) pre_b<false>(A.P, it.u, r);
+            asm volatile("griddepcontrol.wait;" ::: "memory");
+            asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+            if (it.live) post_b<false>(A.P, it.u, r);
+        }
+        sample(A, (blockIdx.z * A.nby + blockIdx.y) * A.nbx + blockIdx.x, t);
+    }
+}
+
+// running DFTs over the samples of a launch's steps, in step order (the
+// accumulation of probe_update): one warp per (probe, frequency), a step per
+// lane for the phase factors, the sums in sequence
+__global__ void __launch_bounds__(32) k_pass_probes(Probes R, const float* samples, long long level, int steps) {
+    const int pr = blockIdx.x, f = blockIdx.y, ln = threadIdx.x;
+    const long long n = level + ln;
+    double s = 0.0, sc = 0.0, ss = 0.0;
+    const bool live = ln < steps;
+    if (live) {
+        s = (double)samples[ln * TF_MAX_PROBES + pr];
+        if (f == 0 && n < R.cap) R.series[(long long)pr * R.cap + n] = s;
+    }
+    if (f >= R.nfreq[pr]) return;
+    const bool on = live && n >= R.n0[pr];
+    if (on) {
+        double ph = R.fdt[pr * TF_MAX_FREQS + f] * (double)n;
+        ph -= floor(ph);
+        double sn, cs;
+        sincospi(2.0 * ph, &sn, &cs);
+        sc = s * cs;
+        ss = s * sn;
+    }
+    double re = R.re[pr * TF_MAX_FREQS + f], im = R.im[pr * TF_MAX_FREQS + f];
+    const unsigned who = __ballot_sync(0xffffffffu, on);
+    for (int u = 0; u < 32; ++u) {
+        const double a = __shfl_sync(0xffffffffu, sc, u), b = __shfl_sync(0xffffffffu, ss, u);
+        if (who >> u & 1u) {
+            re += a * R.dt;
+            im -= b * R.dt;
+        }
+    }
+    if (ln == 0) {
+        R.re[pr * TF_MAX_FREQS + f] = re;
+        R.im[pr * TF_MAX_FREQS + f] = im;
+    }
+}
+
+// per-face 1/mu of the three components on the padded grid
+__global__ void __launch_bounds__(kFT) k_face_imu(Params P, float* w0, float* w1, float* w2) {
+    const long long t = (long long)blockIdx.x * kFT + threadIdx.x;
+    if (t >= P.plane * P.N[2]) return;
+    const int p[3] = {(int)(t % P.pitch), (int)(t / P.pitch % P.N[1]), (int)(t / P.plane)};
+    const bool in = p[0] < P.N[0];
+    w0[t] = in ? inv_mu_face(P, 0, p) : 0.f;
+    w1[t] = in ? inv_mu_face(P, 1, p) : 0.f;
+    w2[t] = in ? inv_mu_face(P, 2, p) : 0.f;
+}
+
+cudaError_t launch_face_imu(const Params& P, float* const w[3], cudaStream_t st) {
+    const long long n = P.plane * P.N[2];
+    k_face_imu<<<(unsigned)((n + kFT - 1) / kFT), kFT, 0, st>>>(P, w[0], w[1], w[2]);
+    return cudaGetLastError();
+}
+
+// `steps` steps from `level`, two launches each, with the amplitudes amp[step];
+// a launch may start while the one before drains (it waits for it before it
+// reads what that one writes)
+cudaError_t launch_passes(const PassArgs& A, const Probes& R, const PassAmps* amp, long long level, int steps,
+                          cudaStream_t st) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(A.nbx, A.nby, A.nbz);
+    cfg.blockDim = dim3(kFT);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cudaError_t e = cudaSuccess;
+    for (int t = 0; t < steps && e == cudaSuccess; ++t) {
+        cfg.numAttrs = t > 0 ? 1 : 0;   // the first launch waits for whatever the stream holds
+        e = cudaLaunchKernelEx(&cfg, k_pass<false>, A, amp[t], t);
+        cfg.numAttrs = 1;
+        if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, k_pass<true>, A, amp[t], t);
+    }
+    if (e == cudaSuccess && R.n > 0) {
+        k_pass_probes<<<dim3(R.n, TF_MAX_FREQS), 32, 0, st>>>(R, A.samples, level, steps);
+        e = cudaGetLastError();
+    }
+    return e;
+}
+
+}  // namespace tf

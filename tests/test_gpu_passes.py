@@ -1,0 +1,111 @@
+"""Steps in place (a B pass and an E pass per step, what tf_step does on grids
+of up to some 25 million points) give the same bits as the staged single-step
+kernel: fields, probe DFTs and series, on every boundary kind, on rows that
+end inside a thread's four points, with sources and probes at the walls,
+varying mu, both edge rules and split calls, and in any mix with staged steps
+on one handle."""
+import numpy as np
+import pytest
+
+from paper_2305_13419_gb300 import workloads as W
+
+torch = pytest.importorskip("torch")
+pytestmark = [pytest.mark.gpu,
+              pytest.mark.skipif(not torch.cuda.is_available(), reason="needs a CUDA GPU")]
+
+P, C, W_, M = "periodic", "cpml", "pec", "mur"
+# size, boundaries, edge rule, theta, range of mu
+CASES = [
+    ((1, 1, 300), (P, P, M), 0, 1.0, (1.0, 1.0)),
+    ((1, 1, 2), (P, P, M), 0, 1.0, (1.0, 1.0)),
+    ((2, 3, 5), (P, P, P), 1, 0.5, (1.0, 2.0)),
+    ((4, 4, 130), (P, P, M), 0, 1.0, (1.0, 1.0)),
+    ((5, 7, 3), (W_, W_, M), 0, 0.5, (1.0, 2.0)),
+    ((33, 17, 9), (W_, P, W_), 1, 1.0, (1.0, 1.0)),
+    ((66, 34, 33), (C, C, C), 0, 1.0, (1.0, 1.0)),
+    ((67, 33, 30), (C, P, C), 0, 0.5, (1.0, 2.0)),
+    ((70, 29, 31), (P, C, M), 1, 1.0, (1.0, 1.0)),
+    ((131, 21, 18), (W_, C, P), 0, 1.0, (1.0, 1.0)),
+    ((96, 50, 40), (P, P, P), 0, 0.5, (1.0, 1.0)),
+    ((65, 8, 64), (P, W_, C), 0, 1.0, (1.0, 2.0)),
+]
+
+
+def _workload(n, bc, rule, theta, mu):
+    w = W.random_box(n=n, bc=bc, seed=sum(n), theta=theta, mu_range=mu, cpml_cells=max(1, min(4, min(n) // 2)))
+    w.edge_rule = rule
+    f = W.C0 / (20 * w.d[2])
+    hi = w.storage_dims()
+    w.sources = [W.Source(comp=c, lo=(n[0] // 3, 0, n[2] // 2), hi=(n[0] // 3 + 5, n[1], n[2] // 2 + 2), amp=0.3 + c,
+                          kind=c, f=f, t0=3e-16, tw=1e-16) for c in range(3)]
+    pts = [(0, 0, 0), (hi[0] - 1, hi[1] - 1, hi[2] - 1), (n[0] // 2, n[1] // 2, n[2] // 2)]
+    w.probes = [W.Probe(comp=c, p=p, freqs=np.linspace(0.5 * f, 2 * f, 3 + 7 * c), n0=5 * c, series=50)
+                for c, p in enumerate(pts)]
+    return w
+
+
+def _grid(w, staged):
+    from paper_2305_13419_gb300 import twofluid as tf
+    g = tf.Grid.from_workload(w)
+    g.set_two_step(False)
+    if staged:
+        g.set_wait_limit(1 << 21)   # a limit of the handle's own: the staged kernel
+    st = W.random_state(11, w.storage_dims())
+    for c in range(9):
+        g.set_field(c, st[c].astype(np.float32))
+    return g
+
+
+def _same(a, b, w, n):
+    for c in range(9):
+        assert np.array_equal(a.field(c), b.field(c)), c
+    for p in range(len(w.probes)):
+        assert np.array_equal(a.probe_dft(p), b.probe_dft(p)), p
+        assert np.array_equal(a.probe_series(p, n), b.probe_series(p, n)), p
+
+
+@pytest.mark.parametrize("case", CASES, ids=lambda c: "x".join(map(str, c[0])) + "-" + "-".join(c[1]))
+def test_passes_give_the_bits_of_staged_steps(case):
+    w = _workload(*case)
+    ref = _grid(w, True)
+    ref.step(41)
+    ref.sync()
+    for chunks in ([41], [1, 2, 38]):
+        g = _grid(w, False)
+        for n in chunks:
+            g.step(n)
+        g.sync()
+        _same(g, ref, w, 41)
+
+
+def test_passes_with_mu_in_blocks():
+    """mu constant over most tile-planes but not over the grid."""
+    w = _workload((96, 48, 20), (P, P, C), 0, 1.0, (1.0, 2.0))
+    w.eps_r[:], w.sigma[:], w.lambda_L[:] = 2.5, 2e5, 40e-9
+    w.mu_r[:] = 1.7
+    w.mu_r[:, :, :2] = 1.3
+    ref = _grid(w, True)
+    ref.step(15)
+    g = _grid(w, False)
+    g.step(15)
+    _same(g, ref, w, 15)
+
+
+@pytest.mark.parametrize("case", [CASES[6], CASES[8]], ids=["cpml", "mur"])
+def test_passes_and_staged_steps_mix(case):
+    """In place, staged and two-step passes in turn on one handle."""
+    w = _workload(*case)
+    ref = _grid(w, True)
+    ref.step(26)
+    g = _grid(w, False)
+    g.step(5)
+    g.set_wait_limit(1 << 21)
+    g.step(3)
+    g.set_wait_limit(None)
+    g.step(4)
+    g.set_two_step(8)
+    g.step(5)
+    g.set_two_step(False)
+    g.step(9)
+    g.sync()
+    _same(g, ref, w, 26)
