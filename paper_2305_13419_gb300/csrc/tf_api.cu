@@ -131,7 +131,7 @@ Layout layout_of(const tf_grid_desc* d) {
     L.off_order_t = o; o += align_up(sizeof(long long) * (size_t)L.max_t);
     L.off_stats = o;  o += align_up(sizeof(StatPartial) * (size_t)(L.N[2] + 1));
     pass_shape(L, cx, cy);
-    L.off_samples = o; o += align_up(sizeof(float) * kPassSteps * TF_MAX_PROBES);
+    L.off_samples = o; o += align_up(2 * sizeof(float) * kPassSteps * TF_MAX_PROBES);   // two groups of steps
     L.off_misc = o;   o += kAlign;
     L.bytes = o;
     return L;
@@ -167,6 +167,7 @@ struct tf_ctx {
     float* fPB[kFieldBuffers][3][3];   // psi_B [buffer][component][axis]
     int cur, nxt;       // buffers of the current and the next state (the third one is scratch)
     int step_blocks;
+    int sms;            // multiprocessors of the device
     int slots, slots2;  // resident CTAs of the single- and two-step kernels on the device
     // two-step passes: the interior box (tiles [tx0, tx1) x [ty0, ty1), planes [tz0, tz1))
     int box_ok;         // the geometry has a box (two-step passes also need uniform mu)
@@ -471,6 +472,7 @@ tf_status tf_create(const tf_grid_desc* desc, void* dev_workspace, size_t bytes,
         // one resident CTA per slot (no more than the units of work).  A grid
         // with fewer items than slots goes out in kSub-plane pieces.
         const long long slots = (long long)sms * per_sm;
+        h->sms = sms;
         h->slots = (int)slots;
         h->slots2 = sms * per_sm2;
         h->fine = items < slots;
@@ -757,6 +759,90 @@ cudaError_t run_passes(tf_ctx* h, const Sources& S, int64_t nsteps) {
     return cudaSuccess;
 }
 
+// A plane is at most kNarrowQuads quads of points, so that a CTA's window of
+// planes runs many steps by itself (tf_narrow.cu): windows of 8 planes at the
+// widest, 2 or 3 steps per launch.  us a step against the passes, which cost
+// two launches however small the grid is: 16 x 8 x 600 (32 quads) 4.5 / 5.7,
+// 4 x 32 x 400 3.5 / 8.4, 9 x 9 x 1000 5.3 / 7.6, 2 x 2 x 2000 0.75 / 7.6.  CPML
+// memories along x and y are not kept there, nor varying mu.
+bool narrow(const tf_ctx* h) {
+    const int per = (h->L.N[0] + 3) / 4 * h->L.N[1];
+    return per <= kNarrowQuads && h->P.uniform_mu && h->P.L[0] == 0 && h->P.L[1] == 0;
+}
+
+// nsteps steps by the narrow kernel, buffer to buffer
+cudaError_t run_narrow(tf_ctx* h, const Sources& S, int64_t nsteps) {
+    NarrowArgs A;
+    memset(&A, 0, sizeof(A));
+    A.S = S;
+    A.tilemat = h->O.tilemat;
+    A.ntx = h->L.ntx;
+    A.nq = (h->L.N[0] + 3) / 4;
+    A.window = kNarrowThreads / (A.nq * h->L.N[1]);
+    float* const samples = (float*)(h->ws + h->L.off_samples);
+    A.nprobe = h->R.n;
+    for (int p = 0; p < h->R.n; ++p) {
+        for (int a = 0; a < 3; ++a) A.pr[p][a] = h->ppos[p][a];
+        A.pr_comp[p] = h->R.comp[p];
+    }
+    // Steps per launch: as many as kPassSteps while the windows, each a plane
+    // wider on both sides per step, and the CTAs of the DFTs still fit the SMs
+    // at once (one to an SM); at least a quarter of the window
+    const int most = (A.window - 1) / 2, least = A.window / 4 < kPassSteps ? A.window / 4 : kPassSteps;
+    const int dft = (h->R.n * TF_MAX_FREQS + kNarrowThreads / 32 - 1) / (kNarrowThreads / 32);
+    int depth = most < kPassSteps ? most : kPassSteps;
+    while (depth > least && (h->L.N[2] + A.window - 2 * depth - 1) / (A.window - 2 * depth) + dft > h->sms) --depth;
+    // psi_E has one array per component: the third psi_B buffer, which only
+    // two-step passes use (a narrow grid has no box for them), is its other one
+    float* pe[2][2];
+    for (int c = 0; c < 2; ++c) {
+        pe[0][c] = h->P.psiE[c][2];
+        pe[1][c] = h->fPB[2][c][2];
+    }
+    int at = 0, last = 0;
+    cudaError_t e = cudaSuccess;
+    for (int64_t s = 0; s < nsteps && e == cudaSuccess;) {
+        const int m = (int)(nsteps - s < depth ? nsteps - s : depth);
+        A.P = h->P;
+        A.steps = m;
+        A.own = A.window - 2 * m;
+        for (int c = 0; c < 3; ++c) {
+            A.E[c] = h->O.E[c];
+            A.B[c] = h->O.B[c];
+            A.J[c] = h->O.J[c];
+        }
+        for (int c = 0; c < 2; ++c) {
+            A.P.psiE[c][2] = pe[at][c];
+            A.psiE[c] = pe[1 - at][c];
+            A.psiB[c] = h->O.psiB[c][2];
+        }
+        for (int u = 0; u < m; ++u)
+            for (int q = 0; q < h->nsrc; ++q)
+                A.amp[q][u] = (float)(h->src[q].amp * waveform(h->src[q], (double)(h->level + u + 1) * h->dt));
+        A.samples = samples + at * kPassSteps * TF_MAX_PROBES;
+        A.samples_before = samples + (1 - at) * kPassSteps * TF_MAX_PROBES;
+        A.level = h->level;
+        A.chained = s > 0;
+        A.steps_before = s > 0 && h->R.n > 0 ? last : 0;
+        e = launch_narrow(A, h->R, h->stream);
+        last = m;
+        at = 1 - at;
+        const int t = h->cur;
+        h->cur = h->nxt;
+        h->nxt = t;
+        bind(h, h->cur, h->nxt, h->P, h->O);
+        h->level += m;
+        s += m;
+    }
+    if (e == cudaSuccess && h->R.n > 0)   // the last launch's samples
+        e = launch_pass_probes(h->R, A.samples, h->level - last, last, h->stream);
+    if (e == cudaSuccess && at && h->P.L[2] > 0)
+        for (int c = 0; c < 2 && e == cudaSuccess; ++c)
+            e = cudaMemcpyAsync(pe[0][c], pe[1][c], sizeof(float) * (size_t)h->L.total, cudaMemcpyDeviceToDevice,
+                                h->stream);
+    return e;
+}
+
 // Does tf_step run in place (tf_pass.cu)?  Not when two-step passes were
 // asked for, nor under a wait limit of the handle's own (the passes wait for
 // nothing).  us per step in place / single staged steps / two-step passes on
@@ -930,7 +1016,7 @@ tf_status tf_step(tf_handle h, int64_t nsteps) {
     Sources S;
     fill_sources(h, S);
     if (in_place(h)) {
-        TF_CUDA(run_passes(h, S, nsteps));
+        TF_CUDA(narrow(h) ? run_narrow(h, S, nsteps) : run_passes(h, S, nsteps));
         return TF_OK;
     }
     TF_CUDA(refresh_order(h, S));

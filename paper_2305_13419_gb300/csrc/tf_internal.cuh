@@ -365,6 +365,30 @@ struct PassAmps {
 };
 cudaError_t launch_passes(const PassArgs& A, const Probes& R, const PassAmps* amp, long long level, int steps,
                           cudaStream_t st);
+cudaError_t launch_pass_probes(const Probes& R, const float* samples, long long level, int steps, cudaStream_t st);
+
+// Many steps per launch on grids whose x-y cross section is a few quads
+// (tf_narrow.cu): from the current buffer to the next one.
+constexpr int kNarrowThreads = 256;
+constexpr int kNarrowQuads = 32;   // quads of a plane at most
+struct NarrowArgs {
+    Params P;
+    Sources S;
+    float amp[TF_MAX_SOURCES][kPassSteps];   // amp * s(t^{n+1}) by source and step (a constant-cache line holds 16 steps)
+    const float4* tilemat;
+    int ntx;
+    float *E[3], *B[3], *J[3];     // the next buffer
+    float *psiB[2], *psiE[2];      // CPML memories of the z axis (components x, y)
+    int nq;                        // quads of a row
+    int steps, window, own;        // steps; planes of a CTA's window, planes it owns: window - 2 steps
+    int nprobe, pr[TF_MAX_PROBES][3], pr_comp[TF_MAX_PROBES];
+    float* samples;                // [step][probe]
+    long long level;               // level at the first step
+    const float* samples_before;   // the samples of the launch before, if any: steps_before > 0
+    int steps_before;
+    int chained;                   // the launch before in the stream is one of these
+};
+cudaError_t launch_narrow(const NarrowArgs& A, const Probes& R, cudaStream_t st);
 cudaError_t launch_face_imu(const Params& P, float* const w[3], cudaStream_t st);
 
 // launchers (tf_kernels.cu)
