@@ -1410,7 +1410,7 @@ tf_status tf_read_field(tf_handle h, int comp, float* dst, int on_device) {
     if (!h || !dst || comp < 0 || comp > 8) return TF_EINVAL;
     float* out = on_device ? dst : h->scratch;
     const double scale = comp < 3 ? 1.0 : comp < 6 ? 1.0 / kC0 : kEps0 / h->dt;
-    TF_CUDA(launch_read_field(h->P, comp, h->primed, out, scale, h->stream));
+    TF_CUDA(launch_read_field(h->P, comp, h->primed, h->O.tilemat, h->L.ntx, out, scale, h->stream));
     if (!on_device)
         TF_CUDA(cudaMemcpyAsync(dst, out, sizeof(float) * h->L.ndense, cudaMemcpyDeviceToHost, h->stream));
     TF_CUDA(cudaStreamSynchronize(h->stream));

@@ -400,8 +400,8 @@ cudaError_t launch_set_field(const Params& P, int comp, const float* dense, floa
                              cudaStream_t st);
 cudaError_t launch_prime(const Params& P, cudaStream_t st);
 cudaError_t launch_mask_js(const Params& P, cudaStream_t st);
-cudaError_t launch_read_field(const Params& P, int comp, int primed, float* dense, double scale,
-                              cudaStream_t st);
+cudaError_t launch_read_field(const Params& P, int comp, int primed, const float4* tilemat, int ntx, float* dense,
+                              double scale, cudaStream_t st);
 // 4-D TMA view (x, y, z, array index) of `narrays` equally spaced arrays with
 // a box of bx x by x 1 x bf; writes a 128-byte CUtensorMap to out128
 cudaError_t make_tensor_map(void* base, const int N[3], int pitch, size_t array_bytes, int narrays, int bx,

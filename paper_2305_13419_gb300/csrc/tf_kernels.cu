@@ -154,33 +154,64 @@ __global__ void k_prime(Params P) {
     }
 }
 
-__global__ void k_read_field(Params P, int comp, int primed, float* dense, double scale) {
-    const long long tot = (long long)P.N[0] * P.N[1] * P.N[2];
-    const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (t >= tot) return;
-    const int i = (int)(t % P.N[0]);
-    const long long r = t / P.N[0];
-    const int p[3] = {i, (int)(r % P.N[1]), (int)(r / P.N[1])};
-    const long long q = lin(P, p[0], p[1], p[2]);
-    double v;
-    if (comp < 3) {
-        v = P.E[comp][q];
-    } else if (comp < 6) {
-        const int cb = comp - 3;
-        float b = P.B[cb][q];
-        if (primed && upd_B(P, cb, p)) b -= 0.5f * curl_E_peek(P, cb, p, q);
-        v = b;
+// v * scale to FP32's rounding, the scale as an unevaluated sum of two FP32
+// numbers: the product's error enters before the one rounding that counts
+// (against FP64 arithmetic it rounds the other way on one value in some 2^22;
+// three FP32 operations where the FP64 pipe takes 48 cycles per warp)
+__device__ __forceinline__ float scaled(float v, float sh, float sl) {
+    const float p = __fmul_rn(v, sh);
+    return isfinite(p) ? __fadd_rn(p, __fmaf_rn(v, sl, __fmaf_rn(v, sh, -p))) : p;
+}
+
+// integer-level value of component c of E (kKind 0), B (1) or Js (2) at a point
+template <int kKind>
+__device__ __forceinline__ float read_point(const Params& P, int c, int primed, const float4* tilemat, int ntx,
+                                            const int p[3], float sh, float sl) {
+    const int q = (int)lin(P, p[0], p[1], p[2]);
+    if constexpr (kKind == 0) {
+        return P.E[c][q];
+    } else if constexpr (kKind == 1) {
+        float b = P.B[c][q];
+        if (primed && upd_B(P, c, p)) b -= 0.5f * curl_E_peek(P, c, p, q);
+        return scaled(b, sh, sl);
     } else {
-        const int c = comp - 6;
-        float jt = 0.f;   // Js lives on superconducting edges only
-        if (upd_E(P, c, p)) {
-            float eps, st, kt;
-            edge_material(P, c, p, eps, st, kt);
-            if (kt > 0.f) jt = P.J[c][q] + (primed ? 0.5f * kt * P.E[c][q] : 0.f);
-        }
-        v = jt;
+        // Js lives on superconducting edges only: none on a tile-plane of one
+        // other material, nor off the tiles (walls)
+        if (p[0] >= (P.per[0] ? P.N[0] : P.n[0]) || p[1] >= (P.per[1] ? P.N[1] : P.n[1])) return 0.f;
+        const float4 rec = __ldg(tilemat + (long long)((p[1] / kSY) * ntx + p[0] / kSX) * P.N[2] + p[2]);
+        if (!isnan(rec.x) && !(rec.z > 0.f)) return 0.f;
+        const float kt = __ldg(P.cj[c] + q);   // zero on the other edges and on edges no step advances
+        if (!(kt > 0.f)) return 0.f;
+        return scaled(P.J[c][q] + (primed ? 0.5f * kt * P.E[c][q] : 0.f), sh, sl);
     }
-    dense[t] = (float)(v * scale);
+}
+
+// Read-back.  Bound by memory: a warp takes 128 points of a row, four loads of
+// each array in flight per thread.  (It was one thread per point with 64-bit
+// divisions and three FP64 operations a point, 2 FP64 lanes per cycle and SM:
+// nine fields of the 1024 x 512 x 256 CPW took 9.3 ms.)  kRows = false: rows
+// shorter than a warp, points in sequence.
+template <int kKind, bool kRows>
+__global__ void __launch_bounds__(256) k_read_field(Params P, int c, int primed, const float4* tilemat, int ntx,
+                                                    float* dense, float sh, float sl) {
+    if constexpr (kRows) {
+        const int j = blockIdx.y * 8 + threadIdx.y, k = blockIdx.z, i0 = blockIdx.x * 128 + threadIdx.x;
+        if (j >= P.N[1]) return;
+        float* const out = dense + ((long long)k * P.N[1] + j) * P.N[0];
+        float v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int p[3] = {i0 + 32 * u, j, k};
+            if (p[0] < P.N[0]) v[u] = read_point<kKind>(P, c, primed, tilemat, ntx, p, sh, sl);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (i0 + 32 * u < P.N[0]) out[i0 + 32 * u] = v[u];
+    } else {
+        const unsigned t = blockIdx.x * 256u + threadIdx.x, row = t / (unsigned)P.N[0];
+        const int p[3] = {(int)(t - row * (unsigned)P.N[0]), (int)(row % (unsigned)P.N[1]), (int)(row / (unsigned)P.N[1])};
+        if (p[2] < P.N[2]) dense[t] = read_point<kKind>(P, c, primed, tilemat, ntx, p, sh, sl);
+    }
 }
 
 // ------------------------------------------------------------ time step
@@ -218,12 +249,28 @@ cudaError_t launch_prime(const Params& P, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_read_field(const Params& P, int comp, int primed, float* dense, double scale,
-                              cudaStream_t st) {
-    const long long tot = (long long)P.N[0] * P.N[1] * P.N[2];
-    k_read_field<<<blocks_for(tot, 256), 256, 0, st>>>(P, comp, primed, dense, scale);
-    return cudaGetLastError();
+template <int kKind>
+static void read_kernel(const Params& P, int c, int primed, const float4* tilemat, int ntx, float* dense, float sh,
+                        float sl, cudaStream_t st) {
+    if (P.N[0] >= 32 && P.N[1] <= 8 * 65535 && P.N[2] <= 65535) {   // (blockIdx.y and z end there)
+        k_read_field<kKind, true><<<dim3((P.N[0] + 127) / 128, (P.N[1] + 7) / 8, P.N[2]), dim3(32, 8), 0, st>>>(
+            P, c, primed, tilemat, ntx, dense, sh, sl);
+    } else {
+        const long long tot = (long long)P.N[0] * P.N[1] * P.N[2];
+        k_read_field<kKind, false><<<blocks_for(tot, 256), 256, 0, st>>>(P, c, primed, tilemat, ntx, dense, sh, sl);
+    }
 }
 
+cudaError_t launch_read_field(const Params& P, int comp, int primed, const float4* tilemat, int ntx, float* dense,
+                              double scale, cudaStream_t st) {
+    const float sh = (float)scale, sl = (float)(scale - (double)sh);
+    if (comp < 3)
+        read_kernel<0>(P, comp, primed, tilemat, ntx, dense, sh, sl, st);
+    else if (comp < 6)
+        read_kernel<1>(P, comp - 3, primed, tilemat, ntx, dense, sh, sl, st);
+    else
+        read_kernel<2>(P, comp - 6, primed, tilemat, ntx, dense, sh, sl, st);
+    return cudaGetLastError();
+}
 
 }  // namespace tf
