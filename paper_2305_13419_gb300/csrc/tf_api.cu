@@ -68,11 +68,15 @@ tf_status validate(const tf_grid_desc* d) {
 // of 251); then few neighbours outside the item along y and z.
 void pass_shape(Layout& L, int cx, int cy) {
     const int nq = (cx + 3) / 4;
+    L.psa = 0;
+    L.psb = kPassBits;
+    L.psc = 0;
     double best = 1e300;
     for (int a = 0; a <= 4; ++a)
         for (int b = 0; a + b <= kPassBits; ++b) {
             const int c = kPassBits - a - b;
             if (c > 0 && (1 << (c - 1)) >= L.kend) continue;
+            if ((cy - 1) >> b > 65534 || (L.kend - 1) >> c > 65534) continue;   // a launch's y and z end there
             const double full = (double)(((nq - 1) >> a) + 1) * (((cy - 1) >> b) + 1) * (((L.kend - 1) >> c) + 1);
             const double halo = 1.0 + 1.2 / (1 << a) + 0.25 / (1 << b) + 0.25 / (1 << c);
             const double cost = full * halo;
@@ -716,8 +720,8 @@ cudaError_t launch_two_steps(tf_ctx* h, Sources& S, cudaEvent_t* ev) {
     return e;
 }
 
-// nsteps steps in place in the current buffer
-cudaError_t run_passes(tf_ctx* h, const Sources& S, int64_t nsteps) {
+// arguments of the passes over the current buffer
+PassArgs pass_args(const tf_ctx* h, const Sources& S) {
     const Layout& L = h->L;
     PassArgs A;
     memset(&A, 0, sizeof(A));
@@ -745,12 +749,22 @@ cudaError_t run_passes(tf_ctx* h, const Sources& S, int64_t nsteps) {
         A.pr_comp[p] = h->R.comp[p];
         A.pr_q[p] = h->R.q[p];
     }
+    return A;
+}
+
+// nsteps steps in place in the current buffer; hist: arrays that take E after
+// step s at hist + 3 s (nullptr: none)
+cudaError_t run_passes(tf_ctx* h, const Sources& S, int64_t nsteps, float* const* hist = nullptr) {
+    const PassArgs A = pass_args(h, S);
     PassAmps amp[kPassSteps];
+    memset(amp, 0, sizeof(amp));
     for (int64_t s = 0; s < nsteps;) {
         const int m = (int)(nsteps - s < kPassSteps ? nsteps - s : kPassSteps);
-        for (int u = 0; u < m; ++u)
+        for (int u = 0; u < m; ++u) {
             for (int q = 0; q < h->nsrc; ++q)
                 amp[u].a[q] = (float)(h->src[q].amp * waveform(h->src[q], (double)(h->level + u + 1) * h->dt));
+            for (int c = 0; hist && c < 3; ++c) amp[u].hist[c] = hist[3 * (s + u) + c];
+        }
         const cudaError_t e = launch_passes(A, h->R, amp, h->level, m, h->stream);
         if (e != cudaSuccess) return e;
         h->level += m;
@@ -1581,7 +1595,7 @@ AdjLayout adj_layout(const tf_ctx* h, int64_t nsteps, int segment) {
     size_t o = 0;
     A.off_ck = o;    o += A.nck * A.ck;
     A.off_hist = o;  o += 2 * (size_t)(segment + 1) * 3 * fb;   // two segments' E history
-    A.off_state = o; o += (size_t)(9 + 4 * h->L.ncpml_axes + 12) * fb;   // E, B, J, psi, edge and face weights
+    A.off_state = o; o += (size_t)(9 + 4 * h->L.ncpml_axes + 3) * fb;   // E, B, J, psi, cb E
     A.off_grad = o;  o += 6 * align_up(sizeof(double) * (size_t)h->L.total);
     A.bytes = o;
     return A;
@@ -1656,14 +1670,56 @@ tf_status tf_adjoint_run(tf_handle h, int64_t nsteps, int probe, int freq_index,
     const size_t fb = align_up(sizeof(float) * (size_t)h->L.total);
     const size_t gb = align_up(sizeof(double) * (size_t)h->L.total);
     tf_status rc;
-    // forward run, a checkpoint at the start of every segment and at the end
-    // (every segment but the first starts primed)
+    // E history of segment s in buffer s % 2
+    auto hist = [&](int64_t s, int64_t m, int c) {
+        return (float*)(sc + A.off_hist + (((size_t)(s & 1) * (segment + 1) + m) * 3 + c) * fb);
+    };
+    auto seg_len = [&](int64_t s) { return (s + 1) * segment <= nsteps ? segment : nsteps - s * segment; };
+    Sources src;
+    fill_sources(h, src);
+    // the steps of segment s from the state the handle holds, E kept at every level
+    float** const to = (float**)malloc(sizeof(float*) * 3 * (size_t)(segment < nsteps ? segment : nsteps));
+    if (!to) return TF_ENOMEM;
+    struct Free {
+        void* p;
+        ~Free() { free(p); }
+    } to_free{to};
+    auto keep_levels = [&](int64_t s) -> tf_status {
+        const int64_t len = seg_len(s);
+        float* const d0[3] = {hist(s, 0, 0), hist(s, 0, 1), hist(s, 0, 2)};
+        TF_CUDA(launch_copy3(d0, h->P.E, h->L.total, h->stream));
+        if (in_place(h)) {   // the E passes write the history as well
+            if (!h->primed) {
+                TF_CUDA(launch_prime(h->P, h->stream));
+                h->primed = 1;
+            }
+            for (int64_t m = 0; m < len; ++m)
+                for (int c = 0; c < 3; ++c) to[3 * m + c] = hist(s, m + 1, c);
+            TF_CUDA(run_passes(h, src, len, to));
+            return TF_OK;
+        }
+        for (int64_t m = 1; m <= len; ++m) {
+            const tf_status r = tf_step(h, 1);
+            if (r != TF_OK) return r;
+            float* const d[3] = {hist(s, m, 0), hist(s, m, 1), hist(s, m, 2)};
+            TF_CUDA(launch_copy3(d, h->P.E, h->L.total, h->stream));
+        }
+        return TF_OK;
+    };
+    // Forward run.  The last two segments' E goes straight into the two history
+    // buffers; the segments before are recomputed later, from a checkpoint at
+    // the start of each (every segment but the first starts primed).
+    const int64_t first_kept = A.nseg > 2 ? A.nseg - 2 : 0;
     for (int64_t s = 0; s < A.nseg; ++s) {
-        if ((rc = tf_checkpoint_save(h, sc + A.off_ck + s * A.ck, A.ck, 1)) != TF_OK) return rc;
-        const int64_t len = (s + 1) * segment <= nsteps ? segment : nsteps - s * segment;
-        if ((rc = tf_step(h, len)) != TF_OK) return rc;
+        if (s < first_kept) {
+            if ((rc = tf_checkpoint_save(h, sc + A.off_ck + s * A.ck, A.ck, 1)) != TF_OK) return rc;
+            rc = tf_step(h, seg_len(s));
+        } else {
+            rc = keep_levels(s);
+        }
+        if (rc != TF_OK) return rc;
     }
-    if ((rc = tf_checkpoint_save(h, sc + A.off_ck + A.nseg * A.ck, A.ck, 1)) != TF_OK) return rc;
+    if (first_kept > 0 && (rc = tf_checkpoint_save(h, sc + A.off_ck + A.nseg * A.ck, A.ck, 1)) != TF_OK) return rc;
     if ((rc = tf_sync(h)) != TF_OK) return rc;
     // objective J = |X|^2 from the probe's FP64 DFT
     double re[TF_MAX_FREQS], im[TF_MAX_FREQS];
@@ -1700,26 +1756,13 @@ tf_status tf_adjoint_run(tf_handle h, int64_t nsteps, int probe, int freq_index,
                 S.psiE[c][a] = fa();
             }
         }
-        for (int c = 0; c < 3; ++c)
-            for (int a = 0; a < 3; ++a) {
-                S.W[c][a] = S.U[c][a] = nullptr;
-                if (a == c) continue;
-                S.W[c][a] = fa();
-                S.U[c][a] = fa();
-            }
+        for (int c = 0; c < 3; ++c) S.V[c] = fa();
         for (int c = 0; c < 3; ++c) {
             S.gE[c] = (double*)(sc + A.off_grad + (size_t)c * gb);
             S.gK[c] = (double*)(sc + A.off_grad + (size_t)(3 + c) * gb);
         }
     }
-    Sources src;
-    fill_sources(h, src);
     const int64_t n0 = h->R.n0[probe];
-    // E history of segment s in buffer s % 2
-    auto hist = [&](int64_t s, int64_t m, int c) {
-        return (float*)(sc + A.off_hist + (((size_t)(s & 1) * (segment + 1) + m) * 3 + c) * fb);
-    };
-    auto seg_len = [&](int64_t s) { return (s + 1) * segment <= nsteps ? segment : nsteps - s * segment; };
     // The recompute of segment s - 1 (forward steps from its checkpoint,
     // keeping E at every level) runs on a second stream, beside the adjoint
     // steps of segment s on the handle's stream: the two touch different
@@ -1727,29 +1770,28 @@ tf_status tf_adjoint_run(tf_handle h, int64_t nsteps, int probe, int freq_index,
     // buffer).  The recompute's step kernel takes one CTA per SM, leaving
     // the rest of each SM to the adjoint passes.
     AdjStreams X;
-    if (!X.create()) return TF_ECUDA;
+    if (first_kept > 0 && !X.create()) return TF_ECUDA;   // (two segments at most: nothing to recompute)
     cudaStream_t const user = h->stream;
     const int keep_blocks = h->step_blocks;
     auto recompute = [&](int64_t s) -> tf_status {
         h->stream = X.rs;
         h->step_blocks = keep_blocks < X.sms ? keep_blocks : X.sms;
         tf_status r = ckpt_restore_async(h, sc + A.off_ck + s * A.ck, s * segment, s > 0 ? 1 : 0);
-        const int64_t len = seg_len(s);
-        for (int64_t m = 0; r == TF_OK && m <= len; ++m) {
-            float* const dst[3] = {hist(s, m, 0), hist(s, m, 1), hist(s, m, 2)};
-            if (launch_copy3(dst, h->P.E, h->L.total, h->stream) != cudaSuccess) r = TF_ECUDA;
-            else if (m < len) r = tf_step(h, 1);
-        }
+        if (r == TF_OK) r = keep_levels(s);
         if (r == TF_OK && cudaEventRecord(X.evR[s & 1], X.rs) != cudaSuccess) r = TF_ECUDA;
         h->stream = user;
         h->step_blocks = keep_blocks;
         return r;
     };
-    if ((rc = recompute(A.nseg - 1)) != TF_OK) return rc;
+    AdjArgs G;
+    memset(&G, 0, sizeof(G));
+    G.G = pass_args(h, src);
+    G.S = S;
+    G.probe_comp = h->R.comp[probe];
+    G.probe_o = 4u * (unsigned)h->R.q[probe];
     for (int64_t s = A.nseg - 1; s >= 0; --s) {
-        // this segment's history is complete
-        TF_CUDA(cudaStreamWaitEvent(user, X.evR[s & 1], 0));
-        if (s > 0) {   // the previous segment's recompute into the other buffer, once its last reader is done
+        if (s < first_kept) TF_CUDA(cudaStreamWaitEvent(user, X.evR[s & 1], 0));   // this segment's history is complete
+        if (s > 0 && s - 1 < first_kept) {   // the segment before, into the other buffer, once its last reader is done
             if (s + 1 < A.nseg) TF_CUDA(cudaStreamWaitEvent(X.rs, X.evA[(s + 1) & 1], 0));
             if ((rc = recompute(s - 1)) != TF_OK) return rc;
         }
@@ -1757,31 +1799,28 @@ tf_status tf_adjoint_run(tf_handle h, int64_t nsteps, int probe, int freq_index,
         // adjoint steps back through the segment
         for (int64_t m = len - 1; m >= 0; --m) {
             const int64_t n = s * segment + m;
-            AdjStep st;
             for (int c = 0; c < 3; ++c) {
-                st.En[c] = hist(s, m, c);
-                st.En1[c] = hist(s, m + 1, c);
+                G.En[c] = hist(s, m, c);
+                G.En1[c] = hist(s, m + 1, c);
             }
-            st.probe_comp = h->R.comp[probe];
-            st.probe_q = h->R.q[probe];
-            st.probe_src = 0.f;
+            G.probe_src = 0.f;
             if (n >= n0) {   // dJ/dE^n = 2 dt Re(conj(X) exp(-i 2 pi f dt n))
                 double ph = f * h->dt * (double)n;
                 ph -= floor(ph);
                 const double ang = 6.283185307179586476925286766559 * ph;
-                st.probe_src = (float)(seed_scale * 2.0 * h->dt * (xr * cos(ang) - xi * sin(ang)));
+                G.probe_src = (float)(seed_scale * 2.0 * h->dt * (xr * cos(ang) - xi * sin(ang)));
             }
             const double t1 = (double)(n + 1) * h->dt;
-            for (int q = 0; q < h->nsrc; ++q) src.amp[q] = (float)(h->src[q].amp * waveform(h->src[q], t1));
-            TF_CUDA(launch_adjoint_step(h->P, S, src, st, h->O.tilemat, h->L.ntx, h->stream));
+            for (int q = 0; q < h->nsrc; ++q) G.W.a[q] = (float)(h->src[q].amp * waveform(h->src[q], t1));
+            TF_CUDA(launch_adjoint_step(G, m < len - 1, user));
         }
-        TF_CUDA(cudaEventRecord(X.evA[s & 1], user));
+        if (first_kept > 0) TF_CUDA(cudaEventRecord(X.evA[s & 1], user));
     }
-    TF_CUDA(cudaStreamWaitEvent(user, X.evR[0], 0));   // the last recompute (segment 0)
+    if (first_kept > 0) TF_CUDA(cudaStreamWaitEvent(user, X.evR[0], 0));   // the last recompute (segment 0)
     TF_CUDA(launch_adjoint_cells(h->P, S, (float)(kC0 * h->dt), 1.0 / seed_scale, grad_eps, grad_lambda,
                                  h->stream));
     // leave the handle in the state the forward run reached
-    if ((rc = tf_checkpoint_load(h, sc + A.off_ck + A.nseg * A.ck, A.ck, 1)) != TF_OK) return rc;
+    if (first_kept > 0 && (rc = tf_checkpoint_load(h, sc + A.off_ck + A.nseg * A.ck, A.ck, 1)) != TF_OK) return rc;
     TF_CUDA(cudaStreamSynchronize(h->stream));
     return TF_OK;
 }

@@ -362,6 +362,7 @@ struct PassArgs {
 };
 struct PassAmps {
     float a[TF_MAX_SOURCES];                    // amp * s(t^{n+1}) of a step
+    float* hist[3];                             // E^{n+1} goes here as well, if not null
 };
 cudaError_t launch_passes(const PassArgs& A, const Probes& R, const PassAmps* amp, long long level, int steps,
                           cudaStream_t st);
@@ -424,18 +425,19 @@ struct AdjState {
     float* psiE[3][3];
     double* gE[3];       // dJ / d eps_r,e
     double* gK[3];       // dJ / d kt_e
-    float* W[3][3];      // edge weights [e][a] (a != e) the face pass differences
-    float* U[3][3];      // face weights [c][a] (a != c) the edge pass differences
+    float* V[3];         // cb Eh, zero on edges the step leaves alone
 };
-struct AdjStep {
+struct AdjArgs {
+    PassArgs G;            // the grid, its items, materials and sources
+    AdjState S;
+    PassAmps W;            // this step's source amplitudes
     const float* En[3];    // E^n
     const float* En1[3];   // E^{n+1} (with this step's soft sources)
     int probe_comp;        // the objective's derivative dJ/dE^n at the probe point
-    long long probe_q;
+    unsigned probe_o;      // byte offset of that point
     float probe_src;
 };
-cudaError_t launch_adjoint_step(const Params& P, const AdjState& A, const Sources& S, const AdjStep& st,
-                                const float4* tilemat, int ntx, cudaStream_t stream);
+cudaError_t launch_adjoint_step(const AdjArgs& A, bool chained, cudaStream_t stream);
 // copy three float arrays of n elements (n a multiple of 4, 16-byte aligned)
 cudaError_t launch_copy3(float* const dst[3], float* const src[3], long long n, cudaStream_t stream);
 cudaError_t launch_adjoint_cells(const Params& P, const AdjState& A, float dt_c0, double unscale, float* g_eps,

@@ -29,13 +29,6 @@ using namespace dev;
 constexpr int kFT = kPassThreads;
 constexpr int kFMin = 5;   // resident CTAs per SM: 20 warps of 96 registers
 
-// own values that a pass needs and that nobody else writes: read past L1, so
-// that they may be fetched while the pass before is still running elsewhere
-__device__ __forceinline__ Q4 own4(const float* base, unsigned o) {
-    Q4 q;
-    asm volatile("ld.global.cg.v2.u64 {%0, %1}, [%2];" : "=l"(q.v[0]), "=l"(q.v[1]) : "l"((const char*)base + o) : "memory");
-    return q;
-}
 // profile of the x axis at a quad, zero off its slab lanes
 __device__ __forceinline__ Q4 prof_x(const float* pf, const Quad& u) {
     const Q4 z = {{0, 0}};
@@ -274,6 +267,7 @@ __device__ __forceinline__ void post_e(const PassArgs& A, const Quad& u, const P
         nz = fma4(cb, cz, mul4(ca, r.ez));
     }
     const Sources& S = A.S;
+    float* const* hist = W.hist;
     if (S.n > 0 && u.x + 3 >= S.bb_lo[0] && u.x < S.bb_hi[0] && u.j >= S.bb_lo[1] && u.j < S.bb_hi[1] &&
         u.k >= S.bb_lo[2] && u.k < S.bb_hi[2])
         add_src(S, W, u.x, u.j, u.k, nx, ny, nz);
@@ -288,6 +282,11 @@ __device__ __forceinline__ void post_e(const PassArgs& A, const Quad& u, const P
         if (mx) sto(P.E[0], o, nx);
         if (my) sto(P.E[1], o, ny);
         if (mz) sto(P.E[2], o, nz);
+    }
+    if (hist[0]) {   // (what the adjoint reads of it: the advanced edges)
+        sto(hist[0], o, nx);
+        sto(hist[1], o, ny);
+        sto(hist[2], o, nz);
     }
     const Q4 sum = add4(add4(nx, ny), nz);
     if (!isfinite(lo(sum.v[0]) + hi(sum.v[0])) || !isfinite(lo(sum.v[1]) + hi(sum.v[1])))

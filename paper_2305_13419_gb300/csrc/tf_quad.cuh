@@ -130,6 +130,14 @@ __device__ __forceinline__ Q4 ldo(const float* base, unsigned o) { return ld4((c
 __device__ __forceinline__ void sto(float* base, unsigned o, const Q4& q) { st4((float*)((char*)base + o), q); }
 __device__ __forceinline__ float ldf(const float* base, unsigned o) { return *(const float*)((const char*)base + o); }
 
+// own values that a pass needs and that nobody else writes: read past L1, so
+// that they may be fetched while the pass before is still running elsewhere
+__device__ __forceinline__ Q4 own4(const float* base, unsigned o) {
+    Q4 q;
+    asm volatile("ld.global.cg.v2.u64 {%0, %1}, [%2];" : "=l"(q.v[0]), "=l"(q.v[1]) : "l"((const char*)base + o) : "memory");
+    return q;
+}
+
 // running DFT of probe pr at its frequency f over the samples of `steps` steps
 // from `level`, in step order (the accumulation of probe_update), by one warp:
 // a step per lane for the phase factors, then the two sums, one lane each, in
