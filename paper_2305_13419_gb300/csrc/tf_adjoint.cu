@@ -284,9 +284,9 @@ __device__ __forceinline__ void edges(const AdjArgs& A, const Quad& u) {
     }
     // the coefficients that the forward step used
     const bool coef = isnan(rec.x);
-    auto ca = [&](int e) { return coef ? ldo(P.ca[e], o) : all4(rec.x); };
+    auto ca = [&](int e) { return coef ? (rec.y > 0.f ? all4(1.f) : ldo(P.ca[e], o)) : all4(rec.x); };
     auto cb = [&](int e) { return coef ? ldo(P.cb[e], o) : all4(rec.y); };
-    auto cj = [&](int e) { return coef ? ldo(P.cj[e], o) : all4(rec.z); };
+    auto cj = [&](int e) { return coef && rec.z > 0.f ? ldo(P.cj[e], o) : all4(rec.z); };
     const Q4 cbx = cb(0), cby = cb(1), cbz = cb(2);
     const Q4 vx = mul4(cbx, ex), vy = mul4(cby, ey), vz = mul4(cbz, ez);
     if (!kPlain) {   // psi_Eh = bE (psi_Eh' + sE e)

@@ -860,10 +860,10 @@ cudaError_t run_narrow(tf_ctx* h, const Sources& S, int64_t nsteps) {
 // Does tf_step run in place (tf_pass.cu)?  Not when two-step passes were
 // asked for, nor under a wait limit of the handle's own (the passes wait for
 // nothing).  us per step in place / single staged steps / two-step passes on
-// CPW grids: 0.3 M cells 7 / 21 / 68, 2.1 M 43 / 72 / 126, 4 M 72 / 104 / 149,
-// 8 M 132 / 165 / 182, 17 M 251 / 266 / 273, 25 M 373 / 384 / 369, 43 M 640 /
-// 627 / 600: once E and B have left the L2 cache the 72 bytes per point of the
-// two passes cost more than the staged kernels' 48 and 24.
+// CPW grids: 0.3 M cells 7.5 / 21 / 68, 2.1 M 31 / 72 / 126, 4 M 70 / 104 / 149,
+// 8 M 127 / 165 / 182, 17 M 234 / 266 / 273, 33 M 444 / 475 / 448, 43 M 576 /
+// 627 / 600, 57 M 753 / 797 / 755, 134 M 1900 / 1695 / 1512: on large grids the
+// 72 bytes per point of the two passes cost more than two steps' 48.
 bool in_place(const tf_ctx* h) {
     const bool asked = h->two_step_on == 2 && h->box_ok && h->P.uniform_mu;
     return !asked && h->P.wait_polls == kSpinLimit && h->L.total <= kPassPoints;

@@ -114,7 +114,8 @@ struct StepOut {
     float* J[3];
     float* psiB[3][3];
     const float4* tilemat;   // per (tile, plane): {ca, cb, cj, 1/mu} of a uniform-material
-                             // tile-plane, ca = NaN where the material varies
+                             // tile-plane; {NaN, no conductor: ca = 1, superconductor, -}
+                             // where the material varies
     int ntx, nty, nch;       // tiles along x, y; z chunks
     int kend;                // planes iterated: N2 (periodic z) or N2 - 1
     int ecur, bcur;          // index of the current E / B arrays in the field tensor map
@@ -344,7 +345,7 @@ cudaError_t launch_step_advance(int* step, cudaStream_t st);
 // Steps in place by a B pass and an E pass each (tf_pass.cu): the fields are
 // those of the current buffer.
 constexpr int kPassSteps = 32;     // steps per group of launches (probe samples are kept for that many)
-constexpr long long kPassPoints = 24LL << 20;   // padded points of a grid up to which tf_step runs in place
+constexpr long long kPassPoints = 64LL << 20;   // padded points of a grid up to which tf_step runs in place
 constexpr int kPassBits = 7, kPassThreads = 1 << kPassBits;   // threads of an item, a quad of x points each
 struct PassArgs {
     Params P;

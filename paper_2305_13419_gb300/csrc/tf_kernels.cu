@@ -175,11 +175,11 @@ __device__ __forceinline__ float read_point(const Params& P, int c, int primed, 
         if (primed && upd_B(P, c, p)) b -= 0.5f * curl_E_peek(P, c, p, q);
         return scaled(b, sh, sl);
     } else {
-        // Js lives on superconducting edges only: none on a tile-plane of one
-        // other material, nor off the tiles (walls)
+        // Js lives on superconducting edges only: none on a tile-plane
+        // without a superconducting cell, nor off the tiles (walls)
         if (p[0] >= (P.per[0] ? P.N[0] : P.n[0]) || p[1] >= (P.per[1] ? P.N[1] : P.n[1])) return 0.f;
         const float4 rec = __ldg(tilemat + (long long)((p[1] / kSY) * ntx + p[0] / kSX) * P.N[2] + p[2]);
-        if (!isnan(rec.x) && !(rec.z > 0.f)) return 0.f;
+        if (!(rec.z > 0.f)) return 0.f;
         const float kt = __ldg(P.cj[c] + q);   // zero on the other edges and on edges no step advances
         if (!(kt > 0.f)) return 0.f;
         return scaled(P.J[c][q] + (primed ? 0.5f * kt * P.E[c][q] : 0.f), sh, sl);

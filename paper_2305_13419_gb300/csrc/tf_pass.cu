@@ -27,7 +27,8 @@ namespace {
 using namespace dev;
 
 constexpr int kFT = kPassThreads;
-constexpr int kFMin = 5;   // resident CTAs per SM: 20 warps of 96 registers
+// resident CTAs per SM: 24 warps of 80 registers (B), 20 of 96 (E), no spills
+constexpr int kBMin = 6, kEMin = 5;
 
 // profile of the x axis at a quad, zero off its slab lanes
 __device__ __forceinline__ Q4 prof_x(const float* pf, const Quad& u) {
@@ -37,7 +38,7 @@ __device__ __forceinline__ Q4 prof_x(const float* pf, const Quad& u) {
 
 struct PreB {
     Q4 ox, oy, oz;       // B
-    Q4 z0, z1, x0, x1, y0, y1;   // psi_B pairs of the slab axes z, x, y
+    Q4 p0, p1;                   // psi_B pair of the first slab axis of z, x, y (further ones: when they are used)
     float bz, cz, by, cy;        // CPML coefficients of the plane and the row
 };
 template <bool kPlain>
@@ -47,18 +48,18 @@ __device__ __forceinline__ void pre_b(const Params& P, const Quad& u, PreB& r) {
     r.oz = own4(P.B[2], u.o);
     if (kPlain) return;
     if (u.sz) {
-        r.z0 = own4(P.psiB[0][2], u.o);
-        r.z1 = own4(P.psiB[1][2], u.o);
+        r.p0 = own4(P.psiB[0][2], u.o);
+        r.p1 = own4(P.psiB[1][2], u.o);
         r.bz = __ldg(P.pbB[2] + u.k);
         r.cz = __ldg(P.pcB[2] + u.k);
-    }
-    if (u.sx) {
-        r.x0 = own4(P.psiB[1][0], u.o);
-        r.x1 = own4(P.psiB[2][0], u.o);
+    } else if (u.sx) {
+        r.p0 = own4(P.psiB[1][0], u.o);
+        r.p1 = own4(P.psiB[2][0], u.o);
+    } else if (u.sy) {
+        r.p0 = own4(P.psiB[0][1], u.o);
+        r.p1 = own4(P.psiB[2][1], u.o);
     }
     if (u.sy) {
-        r.y0 = own4(P.psiB[0][1], u.o);
-        r.y1 = own4(P.psiB[2][1], u.o);
         r.by = __ldg(P.pbB[1] + u.j);
         r.cy = __ldg(P.pcB[1] + u.j);
     }
@@ -104,19 +105,22 @@ __device__ __forceinline__ void post_b(const Params& P, const Quad& u, const Pre
         const unsigned mx = u.in, my = u.iny ? u.hv : 0u, mz = u.inz ? u.hv : 0u;
         Q4 n1, n2;
         if (u.sz) {
-            psi_new(P.psiB[0][2], P.psiB[1][2], o, all4(r.bz), all4(r.cz), r.z0, r.z1,
+            psi_new(P.psiB[0][2], P.psiB[1][2], o, all4(r.bz), all4(r.cz), r.p0, r.p1,
                     dEy_z, dEx_z, mx, my, n1, n2);
             bx = add4(bx, n1);
             by = sub4(by, n2);
         }
         if (u.sx) {
-            psi_new(P.psiB[1][0], P.psiB[2][0], o, prof_x(P.pbB[0], u), prof_x(P.pcB[0], u), r.x0, r.x1, dEz_x, dEy_x,
+            const Q4 o1 = u.sz ? ldo(P.psiB[1][0], o) : r.p0, o2 = u.sz ? ldo(P.psiB[2][0], o) : r.p1;
+            psi_new(P.psiB[1][0], P.psiB[2][0], o, prof_x(P.pbB[0], u), prof_x(P.pcB[0], u), o1, o2, dEz_x, dEy_x,
                     u.sx & my, u.sx & mz, n1, n2);
             by = add4(by, n1);
             bz = sub4(bz, n2);
         }
         if (u.sy) {
-            psi_new(P.psiB[0][1], P.psiB[2][1], o, all4(r.by), all4(r.cy), r.y0, r.y1,
+            const bool late = u.sz || u.sx;
+            const Q4 o1 = late ? ldo(P.psiB[0][1], o) : r.p0, o2 = late ? ldo(P.psiB[2][1], o) : r.p1;
+            psi_new(P.psiB[0][1], P.psiB[2][1], o, all4(r.by), all4(r.cy), o1, o2,
                     dEz_y, dEx_y, mx, mz, n1, n2);
             bx = sub4(bx, n1);
             bz = add4(bz, n2);
@@ -134,7 +138,7 @@ __device__ __forceinline__ void post_b(const Params& P, const Quad& u, const Pre
 
 struct PreE {
     Q4 ex, ey, ez;               // E
-    Q4 z0, z1, x0, x1, y0, y1;   // psi_E pairs of the slab axes z, x, y
+    Q4 p0, p1;                   // psi_E pair of the first slab axis of z, x, y (further ones: when they are used)
     float bz, cz, by, cy;        // CPML coefficients of the plane and the row
     float4 rec;
 };
@@ -147,18 +151,18 @@ __device__ __forceinline__ void pre_e(const PassArgs& A, const Quad& u, PreE& r)
     r.ez = own4(P.E[2], u.o);
     if (!kPlain) {
         if (u.sz) {
-            r.z0 = own4(P.psiE[0][2], u.o);
-            r.z1 = own4(P.psiE[1][2], u.o);
+            r.p0 = own4(P.psiE[0][2], u.o);
+            r.p1 = own4(P.psiE[1][2], u.o);
             r.bz = __ldg(P.pbE[2] + u.k);
             r.cz = __ldg(P.pcE[2] + u.k);
-        }
-        if (u.sx) {
-            r.x0 = own4(P.psiE[1][0], u.o);
-            r.x1 = own4(P.psiE[2][0], u.o);
+        } else if (u.sx) {
+            r.p0 = own4(P.psiE[1][0], u.o);
+            r.p1 = own4(P.psiE[2][0], u.o);
+        } else if (u.sy) {
+            r.p0 = own4(P.psiE[0][1], u.o);
+            r.p1 = own4(P.psiE[2][1], u.o);
         }
         if (u.sy) {
-            r.y0 = own4(P.psiE[0][1], u.o);
-            r.y1 = own4(P.psiE[2][1], u.o);
             r.by = __ldg(P.pbE[1] + u.j);
             r.cy = __ldg(P.pcE[1] + u.j);
         }
@@ -180,13 +184,7 @@ __device__ __forceinline__ void post_e(const PassArgs& A, const Quad& u, const P
     const Q4 hx_ym = ldo(P.B[0], oy1), hz_ym = ldo(P.B[2], oy1);
     const float hy_p = ldf(P.B[1], op), hz_p = ldf(P.B[2], op);
     // (the first use of the record: every load above is on its way by now)
-    const bool coef = isnan(r.rec.x), sc = coef || r.rec.z > 0.f;   // per-point coefficients; Js advances on the tile-plane
-    Q4 ojx, ojy, ojz;
-    if (sc) {
-        ojx = ldo(P.J[0], o);
-        ojy = ldo(P.J[1], o);
-        ojz = ldo(P.J[2], o);
-    }
+    const bool coef = isnan(r.rec.x), sc = r.rec.z > 0.f;   // per-point coefficients; Js advances on the tile-plane
     Q4 dHz_y, dHy_z, dHx_z, dHz_x, dHy_x, dHx_y;
     if (kPlain || P.uniform_mu) {
         dHz_y = sub4(hz, hz_ym);
@@ -218,25 +216,29 @@ __device__ __forceinline__ void post_e(const PassArgs& A, const Quad& u, const P
     if (!kPlain) {
         Q4 n1, n2;
         if (u.sz) {
-            psi_new(P.psiE[0][2], P.psiE[1][2], o, all4(r.bz), all4(r.cz), r.z0, r.z1,
+            psi_new(P.psiE[0][2], P.psiE[1][2], o, all4(r.bz), all4(r.cz), r.p0, r.p1,
                     dHy_z, dHx_z, mx, my, n1, n2);
             cx = sub4(cx, n1);
             cy = add4(cy, n2);
         }
         if (u.sx) {
-            psi_new(P.psiE[1][0], P.psiE[2][0], o, prof_x(P.pbE[0], u), prof_x(P.pcE[0], u), r.x0, r.x1, dHz_x, dHy_x,
+            const Q4 o1 = u.sz ? ldo(P.psiE[1][0], o) : r.p0, o2 = u.sz ? ldo(P.psiE[2][0], o) : r.p1;
+            psi_new(P.psiE[1][0], P.psiE[2][0], o, prof_x(P.pbE[0], u), prof_x(P.pcE[0], u), o1, o2, dHz_x, dHy_x,
                     u.sx & my, u.sx & mz, n1, n2);
             cy = sub4(cy, n1);
             cz = add4(cz, n2);
         }
         if (u.sy) {
-            psi_new(P.psiE[0][1], P.psiE[2][1], o, all4(r.by), all4(r.cy), r.y0, r.y1,
+            const bool late = u.sz || u.sx;
+            const Q4 o1 = late ? ldo(P.psiE[0][1], o) : r.p0, o2 = late ? ldo(P.psiE[2][1], o) : r.p1;
+            psi_new(P.psiE[0][1], P.psiE[2][1], o, all4(r.by), all4(r.cy), o1, o2,
                     dHz_y, dHx_y, mx, mz, n1, n2);
             cx = add4(cx, n1);
             cz = sub4(cz, n2);
         }
     }
     if (sc) {
+        const Q4 ojx = ldo(P.J[0], o), ojy = ldo(P.J[1], o), ojz = ldo(P.J[2], o);
         Q4 jx, jy, jz;
         if (coef) {
             jx = fma4(ldo(P.cj[0], o), r.ex, ojx);
@@ -257,9 +259,16 @@ __device__ __forceinline__ void post_e(const PassArgs& A, const Quad& u, const P
     }
     Q4 nx, ny, nz;
     if (coef) {
-        nx = fma4(ldo(P.cb[0], o), cx, mul4(ldo(P.ca[0], o), r.ex));
-        ny = fma4(ldo(P.cb[1], o), cy, mul4(ldo(P.ca[1], o), r.ey));
-        nz = fma4(ldo(P.cb[2], o), cz, mul4(ldo(P.ca[2], o), r.ez));
+        const Q4 bx = ldo(P.cb[0], o), by = ldo(P.cb[1], o), bz = ldo(P.cb[2], o);
+        if (r.rec.y > 0.f) {   // no conductor on the tile-plane: ca = 1
+            nx = fma4(bx, cx, r.ex);
+            ny = fma4(by, cy, r.ey);
+            nz = fma4(bz, cz, r.ez);
+        } else {
+            nx = fma4(bx, cx, mul4(ldo(P.ca[0], o), r.ex));
+            ny = fma4(by, cy, mul4(ldo(P.ca[1], o), r.ey));
+            nz = fma4(bz, cz, mul4(ldo(P.ca[2], o), r.ez));
+        }
     } else {
         const Q4 ca = all4(r.rec.x), cb = all4(r.rec.y);
         nx = fma4(cb, cx, mul4(ca, r.ex));
@@ -344,18 +353,22 @@ __device__ __forceinline__ void sample(const PassArgs& A, int blk, int t) {
 }  // namespace
 
 // One pass of one step over the grid (kE: the E pass).  Bound by the latency
-// of its one round of loads on small grids and by memory on large ones: a step
-// of the 512 x 256 x 128 CPW takes 251 us (5.8 TB/s of the 72 bytes per point
-// plus the CPML memories), of the 256 x 128 x 64 CPW 43 us, of a 1 x 1 x 4480
-// column 7 us (two launches).  Quads and 96 registers (20 warps per SM) beat
-// 64 registers and 32 warps (spills: 54 against 52 us on the 256 x 128 x 64
-// CPW); columns of 4 planes per thread took 55 there.
+// of its one round of loads on small grids (two launches, 7.5 us a step on the
+// 128 x 64 x 40 CPW) and by memory on large ones: the 512 x 256 x 128 CPW takes
+// 234 us a step (6.2 TB/s of 72 bytes per point plus the CPML memories), the
+// 256 x 128 x 64 CPW, whose 90 MB nearly stay in L2, 31.  What is spilled goes to
+// L2 and back: with all three slab axes' memories and Js fetched up front the E
+// pass spilled 170 bytes a thread (252 and 43 us); now the first slab axis is
+// fetched early, the others and Js where they are used.  A step of the latter
+// grid took 41 us while its random substrate read ca, cj and Js as well; the
+// tile-planes' records say where ca is 1 and where nothing superconducts.
+// Columns of 4 planes per thread were slower (55 against 52 us then).
 // Launches overlap (programmatic dependent launch): a thread fetches what
 // only its own pass writes -- one step and two launches ago -- before it waits
 // for the launch before.  That launch lets the next one start only once its
 // own wait is over, so the launch before it is complete by then.
 template <bool kE>
-__global__ void __launch_bounds__(kFT, kFMin) k_pass(const __grid_constant__ PassArgs A, const __grid_constant__ PassAmps W, int t) {
+__global__ void __launch_bounds__(kFT, kE ? kEMin : kBMin) k_pass(const __grid_constant__ PassArgs A, const __grid_constant__ PassAmps W, int t) {
     const Item it = item_at(A, blockIdx.x, blockIdx.y, blockIdx.z);
     if (kE) {
         PreE r;

@@ -1055,7 +1055,10 @@ __global__ void __launch_bounds__(kThreads, 2)
 }
 
 // per (tile, plane): are all cells an owned edge or face of the tile-plane
-// touches alike?  Then store {ca, cb, cj, 1/mu}; else ca = NaN
+// touches alike?  Then store {ca, cb, cj, 1/mu}; else ca = NaN, and 1 or 0 for
+// "no conducting cell: ca = 1 on every edge" and "a superconducting cell".
+// (A plane per CTA: tiles that walked their planes one by one took three
+// barriers and a round of loads for each.)
 __global__ void k_tile_materials(Params P, float4* rec, int ntx, int nty) {
     const int bx = blockIdx.x, by = blockIdx.y;
     const int tid = threadIdx.y * blockDim.x + threadIdx.x, nth = blockDim.x * blockDim.y;
@@ -1064,39 +1067,36 @@ __global__ void k_tile_materials(Params P, float4* rec, int ntx, int nty) {
         if (v >= P.n[a]) return P.per[a] ? v - P.n[a] : P.n[a] - 1;
         return v;
     };
-    __shared__ float ref[4];
-    for (int k = 0; k < P.N[2]; ++k) {
+    for (int k = blockIdx.z; k < P.N[2]; k += gridDim.z) {
         const int kz[2] = {cellc(2, k - 1), cellc(2, k)};
-        if (tid == 0) {
-            const long long m = lin(P, cellc(0, bx * kSX - 1), cellc(1, by * kSY - 1), kz[1]);
-            ref[0] = P.eps[m];
-            ref[1] = P.sig[m];
-            ref[2] = P.kap[m];
-            ref[3] = P.mu[m];
-        }
-        __syncthreads();
-        bool same = true;
+        const long long m0 = lin(P, cellc(0, bx * kSX - 1), cellc(1, by * kSY - 1), kz[1]);
+        const float e0 = P.eps[m0], s0 = P.sig[m0], k0 = P.kap[m0], u0 = P.mu[m0];
+        bool same = true, cond = false, super = false;
         // cells x0-1 .. x0+kSX-1, y0-1 .. y0+kSY-1 (the tile plus its low halo), planes k-1 and k
         for (int t = tid; t < (kSX + 1) * (kSY + 1); t += nth) {
             const int cx = cellc(0, bx * kSX - 1 + t % (kSX + 1)), cy = cellc(1, by * kSY - 1 + t / (kSX + 1));
 #pragma unroll
             for (int z = 0; z < 2; ++z) {
                 const long long m = lin(P, cx, cy, kz[z]);
-                same &= P.eps[m] == ref[0] && P.sig[m] == ref[1] && P.kap[m] == ref[2] && P.mu[m] == ref[3];
+                const float e = P.eps[m], s = P.sig[m], kp = P.kap[m];
+                same &= e == e0 && s == s0 && kp == k0 && P.mu[m] == u0;
+                cond |= s != 0.f;
+                super |= kp != 0.f;
             }
         }
         same = __syncthreads_and(same);
+        cond = __syncthreads_or(cond);
+        super = __syncthreads_or(super);
         if (tid == 0) {
             float4 r;
             if (same) {
-                const float den = ref[0] + P.theta * ref[1];
-                r = make_float4((ref[0] - (1.f - P.theta) * ref[1]) / den, 1.f / den, ref[2], 1.f / ref[3]);
+                const float den = e0 + P.theta * s0;
+                r = make_float4((e0 - (1.f - P.theta) * s0) / den, 1.f / den, k0, 1.f / u0);
             } else {
-                r = make_float4(__int_as_float(0x7fc00000), 0.f, 0.f, 0.f);
+                r = make_float4(__int_as_float(0x7fc00000), cond ? 0.f : 1.f, super ? 1.f : 0.f, 0.f);
             }
             rec[(long long)(by * ntx + bx) * P.N[2] + k] = r;
         }
-        __syncthreads();
     }
 }
 
@@ -1269,7 +1269,7 @@ cudaError_t launch_item_order(const Params& P, const StepOut& O, const Sources& 
 }
 
 cudaError_t launch_tile_materials(const Params& P, float4* rec, int ntx, int nty, cudaStream_t st) {
-    k_tile_materials<<<dim3(ntx, nty), dim3(32, 8), 0, st>>>(P, rec, ntx, nty);
+    k_tile_materials<<<dim3(ntx, nty, P.N[2] < 65535 ? P.N[2] : 65535), dim3(32, 8), 0, st>>>(P, rec, ntx, nty);
     return cudaGetLastError();
 }
 

@@ -1,5 +1,5 @@
 """Steps in place (a B pass and an E pass per step, what tf_step does on grids
-of up to some 25 million points) and many steps per launch (grids with a
+of up to some 65 million points) and many steps per launch (grids with a
 narrow cross section) give the same bits as the staged single-step
 kernel: fields, probe DFTs and series, on every boundary kind, on rows that
 end inside a thread's four points, with sources and probes at the walls,
