@@ -233,15 +233,17 @@ tf_status tf_set_wait_limit(tf_handle h, int64_t polls);
  * returns after enqueueing (use tf_sync per handle). */
 tf_status tf_batch_step(const tf_handle* hs, int n, int64_t nsteps);
 
-/* One launch per step over every grid of a batch (many resonator variants
- * of uneven sizes): the work items of all grids form one list (each grid's
- * own items, the grid's index in the descriptor; the items with CPML
- * corners, sources or Mur planes of every grid first) that the single-step
- * kernel's CTAs share through one counter, each item run with its grid's
- * arguments; 64 steps at a time are captured in a CUDA graph and replayed
- * (the step number lives on the device and a one-thread launch advances it
- * after each step).  Every grid ends with the same bits as tf_step (single
- * steps) would give it.
+/* Advance a batch of grids (many resonator variants of uneven sizes).  Where
+ * every grid may step in place (see tf_step), the grids run one after the
+ * other, a group of steps at a time, on a few streams of the library's.
+ * Otherwise one launch per step runs over every grid: the work items of all
+ * grids form one list (each grid's own items, the grid's index in the
+ * descriptor; the items with CPML corners, sources or Mur planes of every
+ * grid first) that the single-step kernel's CTAs share through one counter,
+ * each item run with its grid's arguments; 64 steps at a time are captured in
+ * a CUDA graph and replayed (the step number lives on the device and a
+ * one-thread launch advances it after each step).  Every grid ends with the
+ * same bits as tf_step (single steps) would give it.
  *   hs, n      handles (distinct, n <= 32768); the run is issued on hs[0]'s
  *              stream after every handle's stream has been synchronised, and
  *              synchronises it;

@@ -1155,6 +1155,75 @@ tf_status batch_check(const tf_handle* hs, int n, int64_t nsteps) {
 
 }  // namespace
 
+namespace {
+
+// Streams of a batch that runs in place.  One, where a grid fills the SMs and
+// its fields stay in L2 while it runs a group of steps by itself; two, where
+// smaller grids leave room, or larger ones ends to fill; four for the smallest.
+// us per step of the batch on 1 / 2 / 4 streams: 16 grids of 2.4 M cells on
+// average 575 / 598 / 628, 8 of 6 M 824 / 774 / 783, 24 of 0.6 M 278 / 182 / 232,
+// 32 of 0.17 M 244 / 140 / 114 (with CTAs of one launch over the whole batch,
+// staged planes: 820, 1070, 504, 320; 200 grids of 36^3 cells: 1217 against 769).
+constexpr int kBatchStreams = 4;
+int batch_streams(const tf_handle* hs, int n) {
+    long long pts = 0;
+    for (int i = 0; i < n; ++i) pts += hs[i]->L.total;
+    pts /= n;
+    return pts < 400000 ? kBatchStreams : pts < 1200000 || pts > 4500000 ? 2 : 1;
+}
+struct BatchStreams {
+    cudaStream_t s[kBatchStreams] = {};
+    int n = 0;
+    bool create(int want) {
+        for (; n < want; ++n)
+            if (cudaStreamCreateWithFlags(&s[n], cudaStreamNonBlocking) != cudaSuccess) return false;
+        return true;
+    }
+    bool sync() {
+        bool ok = true;
+        for (int i = 0; i < n; ++i) ok = cudaStreamSynchronize(s[i]) == cudaSuccess && ok;
+        return ok;
+    }
+    ~BatchStreams() {
+        sync();
+        for (int i = 0; i < n; ++i) cudaStreamDestroy(s[i]);
+    }
+};
+
+// a batch runs grid by grid where every grid may step in place
+bool batch_in_place(const tf_handle* hs, int n) {
+    for (int i = 0; i < n; ++i)
+        if (hs[i]->P.wait_polls != kSpinLimit || hs[i]->L.total > kPassPoints) return false;
+    return true;
+}
+
+// nsteps steps of every grid, a group of launches per grid in turn
+tf_status batch_passes(const tf_handle* hs, int n, int64_t nsteps) {
+    BatchStreams X;
+    if (!X.create(batch_streams(hs, n))) return TF_ECUDA;
+    cudaError_t e = cudaSuccess;
+    for (int64_t s = 0; s < nsteps && e == cudaSuccess; s += kPassSteps) {
+        const int64_t m = nsteps - s < kPassSteps ? nsteps - s : kPassSteps;
+        for (int i = 0; i < n && e == cudaSuccess; ++i) {
+            tf_ctx* h = hs[i];
+            cudaStream_t const own = h->stream;
+            h->stream = X.s[i % X.n];
+            if (!h->primed) {
+                e = launch_prime(h->P, h->stream);
+                h->primed = 1;
+            }
+            Sources S;
+            fill_sources(h, S);
+            if (e == cudaSuccess) e = narrow(h) ? run_narrow(h, S, m) : run_passes(h, S, m);
+            h->stream = own;
+        }
+    }
+    const bool done = X.sync();
+    return e == cudaSuccess && done ? TF_OK : TF_ECUDA;
+}
+
+}  // namespace
+
 tf_status tf_batch_scratch_size(const tf_handle* hs, int n, int64_t nsteps, size_t* bytes) {
     tf_status rc = batch_check(hs, n, nsteps);
     if (rc != TF_OK) return rc;
@@ -1173,6 +1242,7 @@ tf_status tf_batch_run(const tf_handle* hs, int n, int64_t nsteps, void* scratch
     if (n > (1 << 15)) return TF_ENOTSUP;   // the grid index fills descriptor bits 48-62
     // the grids' earlier work is done before the batch reads their state
     for (int i = 0; i < n; ++i) TF_CUDA(cudaStreamSynchronize(hs[i]->stream));
+    if (batch_in_place(hs, n)) return batch_passes(hs, n, nsteps);
     cudaStream_t st = hs[0]->stream;
     const int slots = hs[0]->slots;
     BatchGrid* G = (BatchGrid*)calloc((size_t)n, sizeof(BatchGrid));

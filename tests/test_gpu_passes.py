@@ -119,3 +119,22 @@ def test_passes_and_staged_steps_mix(case):
     g.step(9)
     g.sync()
     _same(g, ref, w, 26)
+
+
+@pytest.mark.parametrize("sizes,count", [((24, 33, 40), 5), ((96, 104), 2)])
+def test_batches_in_place_and_staged(sizes, count):
+    """tf_batch_run grid by grid in place against its one launch per step over
+    all grids, sources and probes and a narrow grid among them."""
+    from paper_2305_13419_gb300 import twofluid as tf
+    ws = [_workload((n, sizes[0] + i, sizes[-1] - i), (C, P, C), 0, 1.0, (1.0, 1.0))
+          for i, n in enumerate((sizes * count)[:count])]
+    ws.append(_workload((2, 3, 40), (P, P, M), 0, 1.0, (1.0, 1.0)))
+    runs = []
+    for staged in (False, True):
+        grids = [_grid(w, staged) for w in ws]
+        tf.batch_run(grids, 35)
+        tf.batch_run(grids, 6)
+        runs.append(grids)
+    for w, a, b in zip(ws, *runs):
+        assert a.level == 41
+        _same(a, b, w, 41)
