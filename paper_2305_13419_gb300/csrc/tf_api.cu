@@ -739,6 +739,7 @@ PassArgs pass_args(const tf_ctx* h, const Sources& S) {
     A.cx = h->P.per[0] ? h->P.N[0] : h->P.n[0];
     A.cy = h->P.per[1] ? h->P.N[1] : h->P.n[1];
     A.kend = L.kend;
+    A.sms = h->sms;
     A.samples = (float*)(h->ws + L.off_samples);
     A.nprobe = h->R.n;
     const int last[3] = {A.cx - 1, A.cy - 1, A.kend - 1};

@@ -356,6 +356,7 @@ struct PassArgs {
     int sa, sb, sc;                             // an item: 2^sa quads x 2^sb rows x 2^sc planes
     int nbx, nby, nbz;                          // items along x, y, z
     int cx, cy, kend;                           // points advanced along x, y, z: [0, c)
+    int sms;                                    // multiprocessors of the device
     int nprobe;
     int pr_block[TF_MAX_PROBES], pr_comp[TF_MAX_PROBES];   // the item that samples a probe
     long long pr_q[TF_MAX_PROBES];

@@ -27,8 +27,8 @@ namespace {
 using namespace dev;
 
 constexpr int kFT = kPassThreads;
-// resident CTAs per SM: 24 warps of 80 registers (B), 20 of 96 (E), no spills
-constexpr int kBMin = 6, kEMin = 5;
+// resident CTAs per SM: 24 warps of 80 registers (B), 20 of 96 (E), 16 of 128 (kEarly), no spills
+constexpr int kBMin = 6, kEMin = 5, kEarlyMin = 4;
 
 // profile of the x axis at a quad, zero off its slab lanes
 __device__ __forceinline__ Q4 prof_x(const float* pf, const Quad& u) {
@@ -38,15 +38,15 @@ __device__ __forceinline__ Q4 prof_x(const float* pf, const Quad& u) {
 
 struct PreB {
     Q4 ox, oy, oz;       // B
-    Q4 p0, p1;                   // psi_B pair of the first slab axis of z, x, y (further ones: when they are used)
+    Q4 p0, p1;                   // psi_B pair of the first slab axis of z, x, y
+    Q4 x0, x1, y0, y1, fb, fc;   // kEarly: the pairs of x and y and the x profiles (else when they are used)
     float bz, cz, by, cy;        // CPML coefficients of the plane and the row
 };
-template <bool kPlain>
+template <bool kEarly>
 __device__ __forceinline__ void pre_b(const Params& P, const Quad& u, PreB& r) {
     r.ox = own4(P.B[0], u.o);
     r.oy = own4(P.B[1], u.o);
     r.oz = own4(P.B[2], u.o);
-    if (kPlain) return;
     if (u.sz) {
         r.p0 = own4(P.psiB[0][2], u.o);
         r.p1 = own4(P.psiB[1][2], u.o);
@@ -63,6 +63,20 @@ __device__ __forceinline__ void pre_b(const Params& P, const Quad& u, PreB& r) {
         r.by = __ldg(P.pbB[1] + u.j);
         r.cy = __ldg(P.pcB[1] + u.j);
     }
+    if (kEarly) {
+        if (u.sx) {
+            r.fb = prof_x(P.pbB[0], u);
+            r.fc = prof_x(P.pcB[0], u);
+            if (u.sz) {
+                r.x0 = own4(P.psiB[1][0], u.o);
+                r.x1 = own4(P.psiB[2][0], u.o);
+            }
+        }
+        if (u.sy && (u.sz || u.sx)) {
+            r.y0 = own4(P.psiB[0][1], u.o);
+            r.y1 = own4(P.psiB[2][1], u.o);
+        }
+    }
 }
 // CPML memory pair: n = b psi + c d, stored on the lanes of m
 __device__ __forceinline__ void psi_new(float* w1, float* w2, unsigned o, const Q4& b, const Q4& c, const Q4& o1,
@@ -74,24 +88,21 @@ __device__ __forceinline__ void psi_new(float* w1, float* w2, unsigned o, const 
     st4m((float*)((char*)w2 + o), n2, o2, m2);
 }
 
-template <bool kPlain>
+template <bool kEarly>
 __device__ __forceinline__ void post_b(const Params& P, const Quad& u, const PreB& r) {
     const unsigned o = u.o, row = 4u * (unsigned)P.pitch, pl = 4u * (unsigned)P.plane;
     unsigned oy1 = o + row, oz1 = o + pl, on = o + 16u;
-    bool wrap = false;
-    if (!kPlain) {
-        if (u.j + 1 == P.N[1]) oy1 = o - (unsigned)u.j * row;
-        if (u.k + 1 == P.N[2]) oz1 = o - (unsigned)u.k * pl;
-        // the point past the quad; at the row's end the wrap to x = 0 (on a walled axis: nothing keeps it)
-        if (u.x + 4 >= P.N[0]) on = o - 4u * (unsigned)u.x;
-        wrap = P.per[0] && u.x + 4 > P.N[0];
-    }
+    if (u.j + 1 == P.N[1]) oy1 = o - (unsigned)u.j * row;
+    if (u.k + 1 == P.N[2]) oz1 = o - (unsigned)u.k * pl;
+    // the point past the quad; at the row's end the wrap to x = 0 (on a walled axis: nothing keeps it)
+    if (u.x + 4 >= P.N[0]) on = o - 4u * (unsigned)u.x;
+    const bool wrap = P.per[0] && u.x + 4 > P.N[0];
     const Q4 ex = ldo(P.E[0], o), ey = ldo(P.E[1], o), ez = ldo(P.E[2], o);
     const Q4 ex_y = ldo(P.E[0], oy1), ez_y = ldo(P.E[2], oy1);
     const Q4 ex_z = ldo(P.E[0], oz1), ey_z = ldo(P.E[1], oz1);
     const float ey_n = ldf(P.E[1], on), ez_n = ldf(P.E[2], on);
     Q4 ey_x = up4(ey, ey_n), ez_x = up4(ez, ez_n);
-    if (!kPlain && wrap) {   // the row ends inside the quad: its last point wraps
+    if (wrap) {   // the row ends inside the quad: its last point wraps
         ey_x = set_lane(ey_x, P.N[0] - 1 - u.x, ey_n);
         ez_x = set_lane(ez_x, P.N[0] - 1 - u.x, ez_n);
     }
@@ -101,35 +112,36 @@ __device__ __forceinline__ void post_b(const Params& P, const Quad& u, const Pre
     Q4 bx = fma4(r2, dEy_z, sub4(r.ox, mul4(r1, dEz_y)));
     Q4 by = fma4(r0, dEz_x, sub4(r.oy, mul4(r2, dEx_z)));
     Q4 bz = fma4(r1, dEx_y, sub4(r.oz, mul4(r0, dEy_x)));
-    if (!kPlain) {
-        const unsigned mx = u.in, my = u.iny ? u.hv : 0u, mz = u.inz ? u.hv : 0u;
-        Q4 n1, n2;
-        if (u.sz) {
-            psi_new(P.psiB[0][2], P.psiB[1][2], o, all4(r.bz), all4(r.cz), r.p0, r.p1,
-                    dEy_z, dEx_z, mx, my, n1, n2);
-            bx = add4(bx, n1);
-            by = sub4(by, n2);
-        }
-        if (u.sx) {
-            const Q4 o1 = u.sz ? ldo(P.psiB[1][0], o) : r.p0, o2 = u.sz ? ldo(P.psiB[2][0], o) : r.p1;
-            psi_new(P.psiB[1][0], P.psiB[2][0], o, prof_x(P.pbB[0], u), prof_x(P.pcB[0], u), o1, o2, dEz_x, dEy_x,
-                    u.sx & my, u.sx & mz, n1, n2);
-            by = add4(by, n1);
-            bz = sub4(bz, n2);
-        }
-        if (u.sy) {
-            const bool late = u.sz || u.sx;
-            const Q4 o1 = late ? ldo(P.psiB[0][1], o) : r.p0, o2 = late ? ldo(P.psiB[2][1], o) : r.p1;
-            psi_new(P.psiB[0][1], P.psiB[2][1], o, all4(r.by), all4(r.cy), o1, o2,
-                    dEz_y, dEx_y, mx, mz, n1, n2);
-            bx = sub4(bx, n1);
-            bz = add4(bz, n2);
-        }
-        if (!u.full) {
-            bx = sel4(bx, r.ox, mx);
-            by = sel4(by, r.oy, my);
-            bz = sel4(bz, r.oz, mz);
-        }
+    const unsigned mx = u.in, my = u.iny ? u.hv : 0u, mz = u.inz ? u.hv : 0u;
+    Q4 n1, n2;
+    if (u.sz) {
+        psi_new(P.psiB[0][2], P.psiB[1][2], o, all4(r.bz), all4(r.cz), r.p0, r.p1,
+                dEy_z, dEx_z, mx, my, n1, n2);
+        bx = add4(bx, n1);
+        by = sub4(by, n2);
+    }
+    if (u.sx) {
+        const Q4 o1 = !u.sz ? r.p0 : kEarly ? r.x0 : ldo(P.psiB[1][0], o);
+        const Q4 o2 = !u.sz ? r.p1 : kEarly ? r.x1 : ldo(P.psiB[2][0], o);
+        const Q4 fb = kEarly ? r.fb : prof_x(P.pbB[0], u), fc = kEarly ? r.fc : prof_x(P.pcB[0], u);
+        psi_new(P.psiB[1][0], P.psiB[2][0], o, fb, fc, o1, o2, dEz_x, dEy_x,
+                u.sx & my, u.sx & mz, n1, n2);
+        by = add4(by, n1);
+        bz = sub4(bz, n2);
+    }
+    if (u.sy) {
+        const bool late = u.sz || u.sx;
+        const Q4 o1 = !late ? r.p0 : kEarly ? r.y0 : ldo(P.psiB[0][1], o);
+        const Q4 o2 = !late ? r.p1 : kEarly ? r.y1 : ldo(P.psiB[2][1], o);
+        psi_new(P.psiB[0][1], P.psiB[2][1], o, all4(r.by), all4(r.cy), o1, o2,
+                dEz_y, dEx_y, mx, mz, n1, n2);
+        bx = sub4(bx, n1);
+        bz = add4(bz, n2);
+    }
+    if (!u.full) {
+        bx = sel4(bx, r.ox, mx);
+        by = sel4(by, r.oy, my);
+        bz = sel4(bz, r.oz, mz);
     }
     sto(P.B[0], o, bx);
     sto(P.B[1], o, by);
@@ -138,47 +150,65 @@ __device__ __forceinline__ void post_b(const Params& P, const Quad& u, const Pre
 
 struct PreE {
     Q4 ex, ey, ez;               // E
-    Q4 p0, p1;                   // psi_E pair of the first slab axis of z, x, y (further ones: when they are used)
+    Q4 p0, p1;                   // psi_E pair of the first slab axis of z, x, y
+    Q4 x0, x1, y0, y1, fb, fc;   // kEarly: the pairs of x and y, the x profiles, Js (else when they are used)
+    Q4 jx, jy, jz;
     float bz, cz, by, cy;        // CPML coefficients of the plane and the row
     float4 rec;
 };
-template <bool kPlain>
+template <bool kEarly>
 __device__ __forceinline__ void pre_e(const PassArgs& A, const Quad& u, PreE& r) {
     const Params& P = A.P;
     r.rec = __ldg(A.tilemat + (long long)((u.j / kSY) * A.ntx + u.x / kSX) * P.N[2] + u.k);
     r.ex = own4(P.E[0], u.o);
     r.ey = own4(P.E[1], u.o);
     r.ez = own4(P.E[2], u.o);
-    if (!kPlain) {
-        if (u.sz) {
-            r.p0 = own4(P.psiE[0][2], u.o);
-            r.p1 = own4(P.psiE[1][2], u.o);
-            r.bz = __ldg(P.pbE[2] + u.k);
-            r.cz = __ldg(P.pcE[2] + u.k);
-        } else if (u.sx) {
-            r.p0 = own4(P.psiE[1][0], u.o);
-            r.p1 = own4(P.psiE[2][0], u.o);
-        } else if (u.sy) {
-            r.p0 = own4(P.psiE[0][1], u.o);
-            r.p1 = own4(P.psiE[2][1], u.o);
+    if (u.sz) {
+        r.p0 = own4(P.psiE[0][2], u.o);
+        r.p1 = own4(P.psiE[1][2], u.o);
+        r.bz = __ldg(P.pbE[2] + u.k);
+        r.cz = __ldg(P.pcE[2] + u.k);
+    } else if (u.sx) {
+        r.p0 = own4(P.psiE[1][0], u.o);
+        r.p1 = own4(P.psiE[2][0], u.o);
+    } else if (u.sy) {
+        r.p0 = own4(P.psiE[0][1], u.o);
+        r.p1 = own4(P.psiE[2][1], u.o);
+    }
+    if (u.sy) {
+        r.by = __ldg(P.pbE[1] + u.j);
+        r.cy = __ldg(P.pcE[1] + u.j);
+    }
+    if (kEarly) {
+        if (u.sx) {
+            r.fb = prof_x(P.pbE[0], u);
+            r.fc = prof_x(P.pcE[0], u);
+            if (u.sz) {
+                r.x0 = own4(P.psiE[1][0], u.o);
+                r.x1 = own4(P.psiE[2][0], u.o);
+            }
         }
-        if (u.sy) {
-            r.by = __ldg(P.pbE[1] + u.j);
-            r.cy = __ldg(P.pcE[1] + u.j);
+        if (u.sy && (u.sz || u.sx)) {
+            r.y0 = own4(P.psiE[0][1], u.o);
+            r.y1 = own4(P.psiE[2][1], u.o);
+        }
+        if (r.rec.z > 0.f) {
+            r.jx = own4(P.J[0], u.o);
+            r.jy = own4(P.J[1], u.o);
+            r.jz = own4(P.J[2], u.o);
         }
     }
 }
 
-template <bool kPlain>
+template <bool kEarly>
 __device__ __forceinline__ void post_e(const PassArgs& A, const Quad& u, const PreE& r, const PassAmps& W) {
     const Params& P = A.P;
     const unsigned o = u.o, row = 4u * (unsigned)P.pitch, pl = 4u * (unsigned)P.plane;
     unsigned oy1 = o - row, oz1 = o - pl, op = o - 4u;
-    if (!kPlain) {   // below a low wall: the own value, whose difference nothing keeps
-        if (u.j == 0) oy1 = P.per[1] ? o + (unsigned)(P.N[1] - 1) * row : o;
-        if (u.k == 0) oz1 = P.per[2] ? o + (unsigned)(P.N[2] - 1) * pl : o;
-        if (u.x == 0) op = P.per[0] ? o + 4u * (unsigned)(P.N[0] - 1) : o;
-    }
+    // below a low wall: the own value, whose difference nothing keeps
+    if (u.j == 0) oy1 = P.per[1] ? o + (unsigned)(P.N[1] - 1) * row : o;
+    if (u.k == 0) oz1 = P.per[2] ? o + (unsigned)(P.N[2] - 1) * pl : o;
+    if (u.x == 0) op = P.per[0] ? o + 4u * (unsigned)(P.N[0] - 1) : o;
     const Q4 hx = ldo(P.B[0], o), hy = ldo(P.B[1], o), hz = ldo(P.B[2], o);
     const Q4 hx_zm = ldo(P.B[0], oz1), hy_zm = ldo(P.B[1], oz1);
     const Q4 hx_ym = ldo(P.B[0], oy1), hz_ym = ldo(P.B[2], oy1);
@@ -186,7 +216,7 @@ __device__ __forceinline__ void post_e(const PassArgs& A, const Quad& u, const P
     // (the first use of the record: every load above is on its way by now)
     const bool coef = isnan(r.rec.x), sc = r.rec.z > 0.f;   // per-point coefficients; Js advances on the tile-plane
     Q4 dHz_y, dHy_z, dHx_z, dHz_x, dHy_x, dHx_y;
-    if (kPlain || P.uniform_mu) {
+    if (P.uniform_mu) {
         dHz_y = sub4(hz, hz_ym);
         dHy_z = sub4(hy, hy_zm);
         dHx_z = sub4(hx, hx_zm);
@@ -211,34 +241,35 @@ __device__ __forceinline__ void post_e(const PassArgs& A, const Quad& u, const P
     Q4 cx = sub4(mul4(r1, dHz_y), mul4(r2, dHy_z));
     Q4 cy = sub4(mul4(r2, dHx_z), mul4(r0, dHz_x));
     Q4 cz = sub4(mul4(r0, dHy_x), mul4(r1, dHx_y));
-    const unsigned mx = kPlain ? 15u : u.iny && u.inz ? u.hv : 0u, my = kPlain ? 15u : u.inz ? u.in : 0u,
-                   mz = kPlain ? 15u : u.iny ? u.in : 0u;
-    if (!kPlain) {
-        Q4 n1, n2;
-        if (u.sz) {
-            psi_new(P.psiE[0][2], P.psiE[1][2], o, all4(r.bz), all4(r.cz), r.p0, r.p1,
-                    dHy_z, dHx_z, mx, my, n1, n2);
-            cx = sub4(cx, n1);
-            cy = add4(cy, n2);
-        }
-        if (u.sx) {
-            const Q4 o1 = u.sz ? ldo(P.psiE[1][0], o) : r.p0, o2 = u.sz ? ldo(P.psiE[2][0], o) : r.p1;
-            psi_new(P.psiE[1][0], P.psiE[2][0], o, prof_x(P.pbE[0], u), prof_x(P.pcE[0], u), o1, o2, dHz_x, dHy_x,
-                    u.sx & my, u.sx & mz, n1, n2);
-            cy = sub4(cy, n1);
-            cz = add4(cz, n2);
-        }
-        if (u.sy) {
-            const bool late = u.sz || u.sx;
-            const Q4 o1 = late ? ldo(P.psiE[0][1], o) : r.p0, o2 = late ? ldo(P.psiE[2][1], o) : r.p1;
-            psi_new(P.psiE[0][1], P.psiE[2][1], o, all4(r.by), all4(r.cy), o1, o2,
-                    dHz_y, dHx_y, mx, mz, n1, n2);
-            cx = add4(cx, n1);
-            cz = sub4(cz, n2);
-        }
+    const unsigned mx = u.iny && u.inz ? u.hv : 0u, my = u.inz ? u.in : 0u, mz = u.iny ? u.in : 0u;
+    Q4 n1, n2;
+    if (u.sz) {
+        psi_new(P.psiE[0][2], P.psiE[1][2], o, all4(r.bz), all4(r.cz), r.p0, r.p1,
+                dHy_z, dHx_z, mx, my, n1, n2);
+        cx = sub4(cx, n1);
+        cy = add4(cy, n2);
+    }
+    if (u.sx) {
+        const Q4 o1 = !u.sz ? r.p0 : kEarly ? r.x0 : ldo(P.psiE[1][0], o);
+        const Q4 o2 = !u.sz ? r.p1 : kEarly ? r.x1 : ldo(P.psiE[2][0], o);
+        const Q4 fb = kEarly ? r.fb : prof_x(P.pbE[0], u), fc = kEarly ? r.fc : prof_x(P.pcE[0], u);
+        psi_new(P.psiE[1][0], P.psiE[2][0], o, fb, fc, o1, o2, dHz_x, dHy_x,
+                u.sx & my, u.sx & mz, n1, n2);
+        cy = sub4(cy, n1);
+        cz = add4(cz, n2);
+    }
+    if (u.sy) {
+        const bool late = u.sz || u.sx;
+        const Q4 o1 = !late ? r.p0 : kEarly ? r.y0 : ldo(P.psiE[0][1], o);
+        const Q4 o2 = !late ? r.p1 : kEarly ? r.y1 : ldo(P.psiE[2][1], o);
+        psi_new(P.psiE[0][1], P.psiE[2][1], o, all4(r.by), all4(r.cy), o1, o2,
+                dHz_y, dHx_y, mx, mz, n1, n2);
+        cx = add4(cx, n1);
+        cz = sub4(cz, n2);
     }
     if (sc) {
-        const Q4 ojx = ldo(P.J[0], o), ojy = ldo(P.J[1], o), ojz = ldo(P.J[2], o);
+        const Q4 ojx = kEarly ? r.jx : ldo(P.J[0], o), ojy = kEarly ? r.jy : ldo(P.J[1], o),
+                 ojz = kEarly ? r.jz : ldo(P.J[2], o);
         Q4 jx, jy, jz;
         if (coef) {
             jx = fma4(ldo(P.cj[0], o), r.ex, ojx);
@@ -280,7 +311,7 @@ __device__ __forceinline__ void post_e(const PassArgs& A, const Quad& u, const P
     if (S.n > 0 && u.x + 3 >= S.bb_lo[0] && u.x < S.bb_hi[0] && u.j >= S.bb_lo[1] && u.j < S.bb_hi[1] &&
         u.k >= S.bb_lo[2] && u.k < S.bb_hi[2])
         add_src(S, W, u.x, u.j, u.k, nx, ny, nz);
-    if (kPlain || u.full) {
+    if (u.full) {
         sto(P.E[0], o, nx);
         sto(P.E[1], o, ny);
         sto(P.E[2], o, nz);
@@ -301,7 +332,7 @@ __device__ __forceinline__ void post_e(const PassArgs& A, const Quad& u, const P
     if (!isfinite(lo(sum.v[0]) + hi(sum.v[0])) || !isfinite(lo(sum.v[1]) + hi(sum.v[1])))
         atomicOr(P.status, kStatusNonFinite);
     // first-order Mur on the z walls: E_w^{n+1} = E_i^n + M (E_i^{n+1} - E_w^n)
-    if (!kPlain && P.bc[2] == TF_BC_MUR && (u.k == 1 || u.k == P.n[2] - 1)) {
+    if (P.bc[2] == TF_BC_MUR && (u.k == 1 || u.k == P.n[2] - 1)) {
         const unsigned wx = u.iny ? u.hv : 0u, wy = u.in;
 #pragma unroll
         for (int w = 0; w < 2; ++w) {
@@ -318,20 +349,8 @@ __device__ __forceinline__ void post_e(const PassArgs& A, const Quad& u, const P
     }
 }
 
-// does an item of points [x0, x1) x [y0, y1) x [z0, z1) stay off the walls, the seams and the CPML slabs?
-__device__ __forceinline__ bool plain_item(const Params& P, int x0, int x1, int y0, int y1, int z0, int z1) {
-    const int a0[3] = {x0, y0, z0}, a1[3] = {x1, y1, z1};
-    bool ok = P.uniform_mu && P.bc[2] != TF_BC_MUR;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        const int lo_ = P.L[a] > 1 ? P.L[a] : 1, hi_ = P.per[a] ? P.N[a] - 1 : P.n[a] - P.L[a];
-        ok = ok && a0[a] >= lo_ && a1[a] <= hi_;
-    }
-    return ok;
-}
-
 struct Item {
-    bool live, plain;
+    bool live;
     Quad u;
 };
 __device__ __forceinline__ Item item_at(const PassArgs& A, int bx, int by, int bz) {
@@ -341,7 +360,6 @@ __device__ __forceinline__ Item item_at(const PassArgs& A, int bx, int by, int b
     const int x0 = 4 * (bx << A.sa), y0 = by << A.sb, z0 = bz << A.sc;
     const int x = x0 + 4 * iq, j = y0 + jr, k = z0 + kr;
     it.live = x < A.cx && j < A.cy && k < A.kend;
-    it.plain = plain_item(A.P, x0, x0 + (4 << A.sa), y0, y0 + (1 << A.sb), z0, z0 + (1 << A.sc));
     it.u = quad_of(A.P, x, j, k);
     return it;
 }
@@ -363,39 +381,32 @@ __device__ __forceinline__ void sample(const PassArgs& A, int blk, int t) {
 // grid took 41 us while its random substrate read ca, cj and Js as well; the
 // tile-planes' records say where ca is 1 and where nothing superconducts.
 // Columns of 4 planes per thread were slower (55 against 52 us then).
+// kEarly fetches every slab axis' memories and Js before the launch before is
+// done; it takes 128 registers, and is used where all CTAs are resident at
+// once all the same: 6.5 against 7.5 us a step on the 96 x 64 x 48 CPW (576
+// items), but 9.2 against 7.6 on the 128 x 64 x 40 one (640 on 608 places).
+// Items off the walls, seams and slabs take the same code: a variant without
+// its tests was no faster.
 // Launches overlap (programmatic dependent launch): a thread fetches what
 // only its own pass writes -- one step and two launches ago -- before it waits
 // for the launch before.  That launch lets the next one start only once its
 // own wait is over, so the launch before it is complete by then.
-template <bool kE>
-__global__ void __launch_bounds__(kFT, kE ? kEMin : kBMin) k_pass(const __grid_constant__ PassArgs A, const __grid_constant__ PassAmps W, int t) {
+template <bool kE, bool kEarly>
+__global__ void __launch_bounds__(kFT, kEarly ? kEarlyMin : kE ? kEMin : kBMin)
+    k_pass(const __grid_constant__ PassArgs A, const __grid_constant__ PassAmps W, int t) {
     const Item it = item_at(A, blockIdx.x, blockIdx.y, blockIdx.z);
-    if (kE) {
+    if constexpr (kE) {
         PreE r;
-        if (it.plain) {
-            pre_e<true>(A, it.u, r);
-            asm volatile("griddepcontrol.wait;" ::: "memory");
-            asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-            post_e<true>(A, it.u, r, W);
-        } else {
-            if (it.live) pre_e<false>(A, it.u, r);
-            asm volatile("griddepcontrol.wait;" ::: "memory");
-            asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-            if (it.live) post_e<false>(A, it.u, r, W);
-        }
+        if (it.live) pre_e<kEarly>(A, it.u, r);
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+        if (it.live) post_e<kEarly>(A, it.u, r, W);
     } else {
         PreB r;
-        if (it.plain) {
-            pre_b<true>(A.P, it.u, r);
-            asm volatile("griddepcontrol.wait;" ::: "memory");
-            asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-            post_b<true>(A.P, it.u, r);
-        } else {
-            if (it.live) pre_b<false>(A.P, it.u, r);
-            asm volatile("griddepcontrol.wait;" ::: "memory");
-            asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-            if (it.live) post_b<false>(A.P, it.u, r);
-        }
+        if (it.live) pre_b<kEarly>(A.P, it.u, r);
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+        if (it.live) post_b<kEarly>(A.P, it.u, r);
         sample(A, (blockIdx.z * A.nby + blockIdx.y) * A.nbx + blockIdx.x, t);
     }
 }
@@ -440,12 +451,16 @@ cudaError_t launch_passes(const PassArgs& A, const Probes& R, const PassAmps* am
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
+    const bool early = A.nbx * A.nby * A.nbz <= kEarlyMin * A.sms;
     cudaError_t e = cudaSuccess;
     for (int t = 0; t < steps && e == cudaSuccess; ++t) {
         cfg.numAttrs = t > 0 ? 1 : 0;   // the first launch waits for whatever the stream holds
-        e = cudaLaunchKernelEx(&cfg, k_pass<false>, A, amp[t], t);
+        e = early ? cudaLaunchKernelEx(&cfg, k_pass<false, true>, A, amp[t], t)
+                  : cudaLaunchKernelEx(&cfg, k_pass<false, false>, A, amp[t], t);
         cfg.numAttrs = 1;
-        if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, k_pass<true>, A, amp[t], t);
+        if (e == cudaSuccess)
+            e = early ? cudaLaunchKernelEx(&cfg, k_pass<true, true>, A, amp[t], t)
+                      : cudaLaunchKernelEx(&cfg, k_pass<true, false>, A, amp[t], t);
     }
     if (e == cudaSuccess && R.n > 0) e = launch_pass_probes(R, A.samples, level, steps, st);
     return e;
