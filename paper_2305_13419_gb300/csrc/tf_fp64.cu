@@ -17,7 +17,10 @@
 // superconducting cells or plain mean; mu on a face: mean of its 2 cells) and
 // the same Roden-Gedney CPML.  It exists to measure how far the FP32 fused
 // step drifts from FP64 arithmetic; the FP64 pipe (1/64 of the FP32 rate on
-// this part) bounds it.
+// this part: 2 lanes per cycle and SM) bounds it, comparisons and conversions
+// included.  So a component's curl and update are six operations in the E
+// launch and four in the B launch where no CPML slab lies (14 and some 9
+// before), and indices and tests of sign stay in the integer pipe.
 #include <math.h>
 #include <stdint.h>
 #include <stdlib.h>
@@ -39,8 +42,12 @@ struct G64 {
     double *E[3], *B[3], *J[3], *Eold[3];
     double *psiB[3][3], *psiE[3][3];
     double *caE[3], *cbE[3], *kapE[3], *imuF[3];   // theta-scheme coefficients of step 3, kappa, 1 / mu_face
-    double *pbE[3], *pcE[3], *pbB[3], *pcB[3];
+    double *pbE[3], *pcE[3], *pbB[3], *pcB[3];   // CPML profiles b and c / d
     const double *eps_c, *mu_c, *kap_c, *sig_c;
+    int uniform_mu;      // mu_r = 1 throughout
+    // products of constants, so that no thread forms them: dt / d (and half of
+    // it), 1 / (mu0 d), dt / 2
+    double dtd[3], hdtd[3], md[3], hdt, imu0;
 };
 
 __device__ __forceinline__ long long ix(const G64& g, int i, int j, int k) {
@@ -49,9 +56,6 @@ __device__ __forceinline__ long long ix(const G64& g, int i, int j, int k) {
 __device__ __forceinline__ long long ci(const G64& g, int i, int j, int k) {
     return ((long long)k * g.n[1] + j) * g.n[0] + i;
 }
-__device__ __forceinline__ int up(const G64& g, int a, int p) { return p + 1 < g.N[a] ? p + 1 : (g.per[a] ? 0 : p); }
-__device__ __forceinline__ int dn(const G64& g, int a, int p) { return p > 0 ? p - 1 : (g.per[a] ? g.N[a] - 1 : p); }
-__device__ __forceinline__ double sgn(int c, int a) { return ((a - c + 3) % 3 == 1) ? 1.0 : -1.0; }
 // component c of E (is_b = false) or B (true) at p is advanced
 __device__ __forceinline__ bool advanced(const G64& g, int c, bool is_b, const int p[3]) {
     for (int a = 0; a < 3; ++a) {
@@ -70,11 +74,21 @@ __device__ __forceinline__ bool slab(const G64& g, int a, int p) {
 }
 __device__ __forceinline__ bool point(const G64& g, long long t, int p[3]) {
     if (t >= g.np) return false;
+    if (g.np <= 0xffffffffll) {   // (64-bit divisions are calls)
+        const unsigned u = (unsigned)t, row = u / (unsigned)g.N[0];
+        p[0] = (int)(u - row * (unsigned)g.N[0]);
+        p[2] = (int)(row / (unsigned)g.N[1]);
+        p[1] = (int)(row - (unsigned)p[2] * (unsigned)g.N[1]);
+        return true;
+    }
     p[0] = (int)(t % g.N[0]);
     p[1] = (int)((t / g.N[0]) % g.N[1]);
     p[2] = (int)(t / ((long long)g.N[0] * g.N[1]));
     return true;
 }
+// is x, which is not negative, above zero (or 1)?  Without the FP64 pipe.
+__device__ __forceinline__ bool above0(double x) { return (__double2hiint(x) | __double2loint(x)) != 0; }
+__device__ __forceinline__ bool is1(double x) { return __double2hiint(x) == 0x3ff00000 && __double2loint(x) == 0; }
 #define POINT_OR_RETURN                                        \
     int p[3];                                                  \
     const long long t = (long long)blockIdx.x * kT + threadIdx.x; \
@@ -130,18 +144,11 @@ __global__ void k64_coeffs(G64 g) {
     }
 }
 
-__device__ __forceinline__ double dE(const G64& g, int e, int a, const int p[3]) {
-    int q[3] = {p[0], p[1], p[2]};
-    q[a] = up(g, a, p[a]);
-    return (g.E[e][ix(g, q[0], q[1], q[2])] - g.E[e][ix(g, p[0], p[1], p[2])]) * g.id[a];
-}
-__device__ __forceinline__ double dH(const G64& g, int h, int a, const int p[3]) {
-    int q[3] = {p[0], p[1], p[2]};
-    q[a] = dn(g, a, p[a]);
-    const long long i0 = ix(g, p[0], p[1], p[2]), i1 = ix(g, q[0], q[1], q[2]);
-    // the two products rounded on their own (no fused multiply-add), so that
-    // equal neighbours give an exact zero as the oracle's divisions do
-    return (__dmul_rn(g.B[h][i0], g.imuF[h][i0]) - __dmul_rn(g.B[h][i1], g.imuF[h][i1])) * g.id[a];
+// difference of E_e along axis a (not divided by the spacing)
+__device__ __forceinline__ double diffE(const G64& g, int e, int a, const int p[3], long long t) {
+    const long long st = a == 0 ? 1 : a == 1 ? g.N[0] : (long long)g.N[0] * g.N[1];
+    const long long q = p[a] + 1 < g.N[a] ? t + st : g.per[a] ? t - (long long)p[a] * st : t;
+    return g.E[e][q] - g.E[e][t];
 }
 
 __global__ void k64_psi_B(G64 g) {
@@ -150,13 +157,14 @@ __global__ void k64_psi_B(G64 g) {
         if (!advanced(g, c, true, p)) continue;
         for (int a = 0; a < 3; ++a)
             if (a != c && g.psiB[c][a] && slab(g, a, p[a]))
-                g.psiB[c][a][t] = g.pbB[a][p[a]] * g.psiB[c][a][t] + g.pcB[a][p[a]] * dE(g, 3 - c - a, a, p);
+                g.psiB[c][a][t] = fma(g.pbB[a][p[a]], g.psiB[c][a][t], g.pcB[a][p[a]] * diffE(g, 3 - c - a, a, p, t));
     }
 }
 
 struct Src64 {
     int n, comp[TF_MAX_SOURCES], lo[TF_MAX_SOURCES][3], hi[TF_MAX_SOURCES][3];
     double v[TF_MAX_SOURCES];
+    int bb_lo[3], bb_hi[3];   // bounding box of all sources
 };
 
 struct Prb64 {
@@ -171,11 +179,12 @@ struct Prb64 {
 // writes):
 //   k64_steps_1_2   probes at level n, step 1 (B half), step 2 (Js half)
 //   k64_step_3_4    step 3 (psi_E, theta step for E), soft sources, step 4
-//                   (Js half with the new E; the Mur walls carry no Js)
-//   k64_steps_5_1_2 step 5 of step n (psi_B at the new E, B half) and, if
-//                   `next`, steps 1 and 2 of step n+1 with the probes at
-//                   level n+1 (E is not written, so both B halves use the
-//                   same curl and psi_B)
+//                   (Js half with the new E; the Mur walls carry no Js) and,
+//                   if `next`, step 2 of step n+1 (the same half again)
+//   k64_steps_5_1   step 5 of step n (psi_B at the new E, B half) and, if
+//                   `next`, step 1 of step n+1 with the probes at level n+1
+//                   (E is not written, so both B halves use the same curl and
+//                   psi_B: one step of dt)
 // Walls of the Mur kind keep E^n of their planes and of the planes next to
 // them in Eold (k64_mur_walls then applies the Mur update).
 __device__ __forceinline__ void keep_mur_old(const G64& g, const int p[3], long long t) {
@@ -197,68 +206,98 @@ __device__ __forceinline__ void probes_at(const G64& g, const Prb64& R, long lon
         }
     }
 }
-__device__ __forceinline__ double curl_E_B(const G64& g, int c, const int p[3], long long t) {
-    double r = 0.0;
-    for (int a = 0; a < 3; ++a) {
-        if (a == c) continue;
-        double v = dE(g, 3 - c - a, a, p);
-        if (g.psiB[c][a]) v += g.psiB[c][a][t];
-        r += sgn(c, a) * v;
+// B_c -= half * curl E (half: dt / 2 or, for two half steps in one, dt; kd: half / d), with
+// the CPML memories as they stand or (kNewPsi) advanced to the E they see
+template <bool kNewPsi>
+__device__ __forceinline__ void update_B(const G64& g, const int p[3], long long t, const double kd[3], double half) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        if (!advanced(g, c, true, p)) continue;
+        // curl_c = + d/da1 E_e1 - d/da2 E_e2
+        const int a1 = (c + 1) % 3, a2 = (c + 2) % 3, e1 = a2, e2 = a1;
+        const double d1 = diffE(g, e1, a1, p, t), d2 = diffE(g, e2, a2, p, t);
+        double b = fma(-kd[a1], d1, fma(kd[a2], d2, g.B[c][t]));
+        // (the slab's memory comes on top, so that a warp with points in and
+        // out of one does not run the update twice)
+        if (g.psiB[c][a1] && slab(g, a1, p[a1])) {
+            double psi = g.psiB[c][a1][t];
+            if (kNewPsi) g.psiB[c][a1][t] = psi = fma(g.pbB[a1][p[a1]], psi, g.pcB[a1][p[a1]] * d1);
+            b = fma(-half, psi, b);
+        }
+        if (g.psiB[c][a2] && slab(g, a2, p[a2])) {
+            double psi = g.psiB[c][a2][t];
+            if (kNewPsi) g.psiB[c][a2][t] = psi = fma(g.pbB[a2][p[a2]], psi, g.pcB[a2][p[a2]] * d2);
+            b = fma(half, psi, b);
+        }
+        g.B[c][t] = b;
     }
-    return r;
 }
 
 __global__ void k64_steps_1_2(G64 g, Prb64 R, long long level) {
     probes_at(g, R, level);
     POINT_OR_RETURN
     keep_mur_old(g, p, t);
+    update_B<false>(g, p, t, g.hdtd, g.hdt);
     for (int c = 0; c < 3; ++c)
-        if (advanced(g, c, true, p)) g.B[c][t] -= 0.5 * g.dt * curl_E_B(g, c, p, t);
-    for (int c = 0; c < 3; ++c)
-        if (advanced(g, c, false, p) && g.kapE[c][t] > 0.0) g.J[c][t] += 0.5 * g.dt * g.kapE[c][t] * g.E[c][t];
+        if (advanced(g, c, false, p) && above0(g.kapE[c][t])) g.J[c][t] += g.hdt * g.kapE[c][t] * g.E[c][t];
 }
 
-__global__ void k64_step_3_4(G64 g, Src64 S) {
+// kUni: mu_r = 1 throughout.  next: step 2 of the next step as well (its Js
+// half step takes the same E).
+template <bool kUni>
+__global__ void __launch_bounds__(kT) k64_step_3_4(G64 g, Src64 S, int next) {
     POINT_OR_RETURN
+    const bool src = S.n > 0 && p[0] >= S.bb_lo[0] && p[0] < S.bb_hi[0] && p[1] >= S.bb_lo[1] && p[1] < S.bb_hi[1] &&
+                     p[2] >= S.bb_lo[2] && p[2] < S.bb_hi[2];
+#pragma unroll
     for (int c = 0; c < 3; ++c) {
         if (!advanced(g, c, false, p)) continue;
-        for (int a = 0; a < 3; ++a)
-            if (a != c && g.psiE[c][a] && slab(g, a, p[a]))
-                g.psiE[c][a][t] = g.pbE[a][p[a]] * g.psiE[c][a][t] + g.pcE[a][p[a]] * dH(g, 3 - c - a, a, p);
-        double r = 0.0;
-        for (int a = 0; a < 3; ++a) {
-            if (a == c) continue;
-            double v = dH(g, 3 - c - a, a, p);
-            if (g.psiE[c][a]) v += g.psiE[c][a][t];
-            r += sgn(c, a) * v;
+        // curl_c = + d/da1 H_h1 - d/da2 H_h2, backward differences
+        const int a1 = (c + 1) % 3, a2 = (c + 2) % 3, h1 = a2, h2 = a1;
+        auto diffH = [&](int h, int a) {
+            const long long st = a == 0 ? 1 : a == 1 ? g.N[0] : (long long)g.N[0] * g.N[1];
+            const long long q = p[a] > 0 ? t - st : g.per[a] ? t + (long long)(g.N[a] - 1) * st : t;
+            // where mu varies: the two products rounded on their own (no fused
+            // multiply-add), so that equal neighbours give an exact zero as
+            // the oracle's divisions do
+            if constexpr (kUni) return g.B[h][t] - g.B[h][q];
+            return __dmul_rn(g.B[h][t], g.imuF[h][t]) - __dmul_rn(g.B[h][q], g.imuF[h][q]);
+        };
+        const double d1 = diffH(h1, a1), d2 = diffH(h2, a2);
+        const double k1 = kUni ? g.md[a1] : g.id[a1], k2 = kUni ? g.md[a2] : g.id[a2];
+        double r = fma(d1, k1, -(d2 * k2));
+        if (g.psiE[c][a1] && slab(g, a1, p[a1])) {
+            const double m = kUni ? g.pcE[a1][p[a1]] * g.imu0 : g.pcE[a1][p[a1]];
+            r += g.psiE[c][a1][t] = fma(g.pbE[a1][p[a1]], g.psiE[c][a1][t], m * d1);
         }
-        double e = g.caE[c][t] * g.E[c][t] + g.cbE[c][t] * (r - g.J[c][t]);
-        for (int s = 0; s < S.n; ++s)
-            if (S.comp[s] == c && p[0] >= S.lo[s][0] && p[0] < S.hi[s][0] && p[1] >= S.lo[s][1] &&
-                p[1] < S.hi[s][1] && p[2] >= S.lo[s][2] && p[2] < S.hi[s][2])
-                e += S.v[s];
+        if (g.psiE[c][a2] && slab(g, a2, p[a2])) {
+            const double m = kUni ? g.pcE[a2][p[a2]] * g.imu0 : g.pcE[a2][p[a2]];
+            r -= g.psiE[c][a2][t] = fma(g.pbE[a2][p[a2]], g.psiE[c][a2][t], m * d2);
+        }
+        const double ca = g.caE[c][t], e0 = g.E[c][t], kap = g.kapE[c][t], js = g.J[c][t];
+        if (above0(fabs(js))) r -= js;
+        double e = fma(g.cbE[c][t], r, is1(ca) ? e0 : ca * e0);
+        if (src)
+            for (int s = 0; s < S.n; ++s)
+                if (S.comp[s] == c && p[0] >= S.lo[s][0] && p[0] < S.hi[s][0] && p[1] >= S.lo[s][1] &&
+                    p[1] < S.hi[s][1] && p[2] >= S.lo[s][2] && p[2] < S.hi[s][2])
+                    e += S.v[s];
         g.E[c][t] = e;
-        if (g.kapE[c][t] > 0.0) g.J[c][t] += 0.5 * g.dt * g.kapE[c][t] * e;
+        if (above0(kap)) {
+            const double x = g.hdt * kap * e;
+            g.J[c][t] = next ? js + x + x : js + x;
+        }
     }
 }
 
-__global__ void k64_steps_5_1_2(G64 g, Prb64 R, long long level_next, int next) {
+__global__ void __launch_bounds__(kT) k64_steps_5_1(G64 g, Prb64 R, long long level_next, int next) {
     if (next) probes_at(g, R, level_next);
     POINT_OR_RETURN
     if (next) keep_mur_old(g, p, t);
-    for (int c = 0; c < 3; ++c) {
-        if (!advanced(g, c, true, p)) continue;
-        for (int a = 0; a < 3; ++a)
-            if (a != c && g.psiB[c][a] && slab(g, a, p[a]))
-                g.psiB[c][a][t] = g.pbB[a][p[a]] * g.psiB[c][a][t] + g.pcB[a][p[a]] * dE(g, 3 - c - a, a, p);
-        const double r = curl_E_B(g, c, p, t);
-        double b = g.B[c][t] - 0.5 * g.dt * r;
-        if (next) b -= 0.5 * g.dt * r;
-        g.B[c][t] = b;
-    }
     if (next)
-        for (int c = 0; c < 3; ++c)
-            if (advanced(g, c, false, p) && g.kapE[c][t] > 0.0) g.J[c][t] += 0.5 * g.dt * g.kapE[c][t] * g.E[c][t];
+        update_B<true>(g, p, t, g.dtd, g.dt);
+    else
+        update_B<true>(g, p, t, g.hdtd, g.hdt);
 }
 
 // the Mur walls (planes 0 and n of z; blockIdx.y picks the wall)
@@ -386,6 +425,13 @@ tf_status tf64_create(const tf_grid_desc* d, void* ws, size_t bytes, tf64_handle
     g.np = L.np;
     g.edge_rule = d->edge_rule;
     g.dt = d->dt > 0 ? d->dt : d->courant / (kC0d * sqrt(1 / (h[0] * h[0]) + 1 / (h[1] * h[1]) + 1 / (h[2] * h[2])));
+    for (int a = 0; a < 3; ++a) {
+        g.dtd[a] = g.dt * g.id[a];
+        g.hdtd[a] = 0.5 * g.dt * g.id[a];
+        g.md[a] = g.id[a] / kMu0d;
+    }
+    g.hdt = 0.5 * g.dt;
+    g.imu0 = 1.0 / kMu0d;
     g.theta = d->theta;
     g.murM = (kC0d * g.dt - h[2]) / (kC0d * g.dt + h[2]);
     char* b = (char*)ws;
@@ -448,7 +494,7 @@ tf_status tf64_create(const tf_grid_desc* d, void* ws, size_t bytes, tf64_handle
                     }
                 }
                 q[2 * half][pp] = bb;
-                q[2 * half + 1][pp] = cc;
+                q[2 * half + 1][pp] = cc * g.id[a];
             }
         g.pbE[a] = prof + (size_t)(4 * a + 0) * nprof;
         g.pcE[a] = prof + (size_t)(4 * a + 1) * nprof;
@@ -478,12 +524,14 @@ tf_status tf64_set_materials(tf64_handle h, const double* eps_r, const double* m
     const long long nc = (long long)g.n[0] * g.n[1] * g.n[2];
     double* hc = (double*)malloc(sizeof(double) * 4 * (size_t)nc);
     if (!hc) return TF_ENOMEM;
+    g.uniform_mu = 1;
     for (long long m = 0; m < nc; ++m) {
         const double e = eps_r ? eps_r[m] : 1.0, u = mu_r ? mu_r[m] : 1.0;
         const double l = lambda_L ? lambda_L[m] : 0.0, s = sigma ? sigma[m] : 0.0;
         if (!(e > 0) || !(u > 0) || !(s >= 0) || l < 0) { free(hc); return TF_EINVAL; }
         hc[m] = e;
         hc[nc + m] = u;
+        if (u != 1.0) g.uniform_mu = 0;
         hc[2 * nc + m] = (l > 0 && isfinite(l)) ? 1.0 / (l * l * kMu0d * u) : 0.0;
         hc[3 * nc + m] = s;
     }
@@ -562,7 +610,12 @@ tf_status tf64_step(tf64_handle h, int64_t nsteps) {
     S.n = h->nsrc;
     for (int s = 0; s < h->nsrc; ++s) {
         S.comp[s] = h->src[s].comp;
-        for (int a = 0; a < 3; ++a) { S.lo[s][a] = h->src[s].lo[a]; S.hi[s][a] = h->src[s].hi[a]; }
+        for (int a = 0; a < 3; ++a) {
+            S.lo[s][a] = h->src[s].lo[a];
+            S.hi[s][a] = h->src[s].hi[a];
+            if (s == 0 || S.lo[s][a] < S.bb_lo[a]) S.bb_lo[a] = S.lo[s][a];
+            if (s == 0 || S.hi[s][a] > S.bb_hi[a]) S.bb_hi[a] = S.hi[s][a];
+        }
     }
     const bool mur = g.bc[2] == TF_BC_MUR;
     const unsigned nbw = (unsigned)(((long long)g.N[0] * g.N[1] + kT - 1) / kT);
@@ -574,10 +627,13 @@ tf_status tf64_step(tf64_handle h, int64_t nsteps) {
         const double t1 = (double)(h->level + 1) * g.dt;
         for (int q = 0; q < h->nsrc; ++q)
             S.v[q] = wave64(h->src[q].kind, h->src[q].amp, h->src[q].f, h->src[q].t0, h->src[q].tw, t1);
-        k64_step_3_4<<<nb, kT, 0, h->st>>>(g, S);
-        if (mur) k64_mur_walls<<<dim3(nbw, 2), kT, 0, h->st>>>(g);
         const int next = s + 1 < nsteps;
-        k64_steps_5_1_2<<<nb, kT, 0, h->st>>>(g, h->R, h->level + 1, next);
+        if (g.uniform_mu)
+            k64_step_3_4<true><<<nb, kT, 0, h->st>>>(g, S, next);
+        else
+            k64_step_3_4<false><<<nb, kT, 0, h->st>>>(g, S, next);
+        if (mur) k64_mur_walls<<<dim3(nbw, 2), kT, 0, h->st>>>(g);
+        k64_steps_5_1<<<nb, kT, 0, h->st>>>(g, h->R, h->level + 1, next);
         C64(cudaGetLastError());
         h->level++;
     }
