@@ -28,6 +28,7 @@ struct Layout {
     int psa, psb, psc, pnbx, pnby, pnbz;   // items of the steps in place: 2^sa quads x 2^sb rows x 2^sc planes
     long long max_s, max_t;   // capacity of the shell and two-step work lists
     long long scratch_floats;
+    int nstat;              // partials of the statistics
 };
 
 double dt_of(const tf_grid_desc* d) {
@@ -133,7 +134,8 @@ Layout layout_of(const tf_grid_desc* d) {
     // box list: its tiles in items of at least kTBLenMin planes
     L.max_t = (long long)L.ntx * L.nty * (L.N[2] / kTBLenMin + 1);
     L.off_order_t = o; o += align_up(sizeof(long long) * (size_t)L.max_t);
-    L.off_stats = o;  o += align_up(sizeof(StatPartial) * (size_t)(L.N[2] + 1));
+    L.nstat = L.N[2] > kStatPartials ? L.N[2] : kStatPartials;
+    L.off_stats = o;  o += align_up(sizeof(StatPartial) * (size_t)(L.nstat + 1));
     pass_shape(L, cx, cy);
     L.off_samples = o; o += align_up(2 * sizeof(float) * kPassSteps * TF_MAX_PROBES);   // two groups of steps
     L.off_misc = o;   o += kAlign;
@@ -1901,8 +1903,8 @@ tf_status tf_field_stats(tf_handle h, int comp, double* sumsq, double* maxabs, i
     const float* f = comp < 3 ? h->P.E[comp] : comp < 6 ? h->P.B[comp - 3] : h->P.J[comp - 6];
     const double scale = comp < 3 ? 1.0 : comp < 6 ? 1.0 / kC0 : kEps0 / h->dt;
     StatPartial* part = (StatPartial*)(h->ws + h->L.off_stats);
-    StatPartial* out = part + h->L.N[2];
-    TF_CUDA(launch_field_stats(f, h->L.N[0], h->L.N[1], h->L.N[2], h->L.pitch, h->P.plane, scale, part, out,
+    StatPartial* out = part + h->L.nstat;
+    TF_CUDA(launch_field_stats(f, h->L.N[0], h->L.N[1], h->L.N[2], h->L.pitch, h->P.plane, scale, part, h->L.nstat, out,
                                h->stream));
     StatPartial r;
     TF_CUDA(cudaMemcpyAsync(&r, out, sizeof(r), cudaMemcpyDeviceToHost, h->stream));

@@ -451,7 +451,8 @@ cudaError_t launch_item_order(const Params& P, const StepOut& O, const Sources& 
                               int* count, cudaStream_t st);
 int step_blocks_per_sm();
 cudaError_t launch_field_stats(const float* f, int n0, int n1, int n2, int pitch, long long plane, double scale,
-                               StatPartial* partials, StatPartial* out, cudaStream_t st);
+                               StatPartial* partials, int capacity, StatPartial* out, cudaStream_t st);
+constexpr int kStatPartials = 1216;   // partials that a grid's scratch holds at least
 cudaError_t launch_fit_q(const double* re, const double* im, const double* fdt, int nfreq,
                          double dt, long long n0, long long N, double f_guess, double q_guess,
                          double* out, cudaStream_t st);
