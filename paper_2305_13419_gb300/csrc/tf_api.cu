@@ -1703,20 +1703,44 @@ struct AdjStreams {
     }
 };
 
+// The adjoint's checkpoints, in its own scratch: the parts to (save) or from a
+// blob, enqueued in one launch where the alignment allows 16-byte accesses (a
+// restore of 21 parts into three buffers each was 63 copies, 2.5 us each on
+// the host, more than the recomputed segment's launches on a small grid).  The
+// public save and load keep one copy per part: those check a caller's range.
+cudaError_t copy_parts(const tf_ctx* h, char* blob, bool save) {
+    CkptPart parts[40];
+    const int n = ckpt_parts(h, parts);
+    CopyParts C;
+    C.n = 0;
+    size_t o = kCkptHeader;
+    cudaError_t e = cudaSuccess;
+    for (int k = 0; k < n && e == cudaSuccess; ++k) {
+        const CkptPart& p = parts[k];
+        if ((uintptr_t)(blob + o) % 16 == 0 && p.bytes % 16 == 0 && C.n < 32) {
+            CopyParts::Part& c = C.part[C.n++];
+            c.n16 = (long long)(p.bytes / 16);
+            c.src = save ? (const void*)p.cur : (const void*)(blob + o);
+            c.dst[0] = save ? (void*)(blob + o) : (void*)p.cur;
+            // the other buffers of a rotating array hold the same values, so that
+            // points the step never writes (walls) agree in all of them
+            for (int b = 0; b < 2; ++b) c.dst[1 + b] = save ? nullptr : (void*)p.other[b];
+        } else {
+            e = cudaMemcpyAsync(save ? blob + o : (char*)p.cur, save ? (const char*)p.cur : blob + o, p.bytes,
+                                cudaMemcpyDeviceToDevice, h->stream);
+            for (int b = 0; b < 2 && !save && e == cudaSuccess; ++b)
+                if (p.other[b])
+                    e = cudaMemcpyAsync(p.other[b], blob + o, p.bytes, cudaMemcpyDeviceToDevice, h->stream);
+        }
+        o += p.bytes;
+    }
+    return e == cudaSuccess ? launch_copy_parts(C, h->sms, h->stream) : e;
+}
+
 // a checkpoint this run wrote (so its header needs no check) back into the
 // grid, enqueued on the handle's stream without waiting for it
 tf_status ckpt_restore_async(tf_ctx* h, const char* src, int64_t level, int primed) {
-    CkptPart parts[40];
-    const int n = ckpt_parts(h, parts);
-    size_t o = kCkptHeader;
-    for (int k = 0; k < n; ++k) {
-        TF_CUDA(cudaMemcpyAsync(parts[k].cur, src + o, parts[k].bytes, cudaMemcpyDeviceToDevice, h->stream));
-        for (int b = 0; b < 2; ++b)
-            if (parts[k].other[b])
-                TF_CUDA(cudaMemcpyAsync(parts[k].other[b], src + o, parts[k].bytes, cudaMemcpyDeviceToDevice,
-                                        h->stream));
-        o += parts[k].bytes;
-    }
+    TF_CUDA(copy_parts(h, (char*)src, false));
     TF_CUDA(cudaMemsetAsync(h->status, 0, sizeof(unsigned), h->stream));
     h->level = level;
     h->primed = primed;
@@ -1785,14 +1809,16 @@ tf_status tf_adjoint_run(tf_handle h, int64_t nsteps, int probe, int freq_index,
     const int64_t first_kept = A.nseg > 2 ? A.nseg - 2 : 0;
     for (int64_t s = 0; s < A.nseg; ++s) {
         if (s < first_kept) {
-            if ((rc = tf_checkpoint_save(h, sc + A.off_ck + s * A.ck, A.ck, 1)) != TF_OK) return rc;
+            TF_CUDA(copy_parts(h, sc + A.off_ck + s * A.ck, true));
             rc = tf_step(h, seg_len(s));
         } else {
             rc = keep_levels(s);
         }
         if (rc != TF_OK) return rc;
     }
-    if (first_kept > 0 && (rc = tf_checkpoint_save(h, sc + A.off_ck + A.nseg * A.ck, A.ck, 1)) != TF_OK) return rc;
+    const int64_t end_level = h->level;
+    const int end_primed = h->primed;
+    if (first_kept > 0) TF_CUDA(copy_parts(h, sc + A.off_ck + A.nseg * A.ck, true));
     if ((rc = tf_sync(h)) != TF_OK) return rc;
     // objective J = |X|^2 from the probe's FP64 DFT
     double re[TF_MAX_FREQS], im[TF_MAX_FREQS];
@@ -1893,7 +1919,9 @@ tf_status tf_adjoint_run(tf_handle h, int64_t nsteps, int probe, int freq_index,
     TF_CUDA(launch_adjoint_cells(h->P, S, (float)(kC0 * h->dt), 1.0 / seed_scale, grad_eps, grad_lambda,
                                  h->stream));
     // leave the handle in the state the forward run reached
-    if (first_kept > 0 && (rc = tf_checkpoint_load(h, sc + A.off_ck + A.nseg * A.ck, A.ck, 1)) != TF_OK) return rc;
+    if (first_kept > 0 &&
+        (rc = ckpt_restore_async(h, sc + A.off_ck + A.nseg * A.ck, end_level, end_primed)) != TF_OK)
+        return rc;
     TF_CUDA(cudaStreamSynchronize(h->stream));
     return TF_OK;
 }

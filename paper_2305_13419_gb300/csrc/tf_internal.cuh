@@ -399,6 +399,16 @@ cudaError_t launch_convert_materials(const Params& P, const float* eps_r, const 
                                      const float* lam, const float* sigma, double dt,
                                      float* eps, float* sig, float* kap, float* mu,
                                      unsigned* minmax, cudaStream_t st);
+// copies of 16-byte aligned parts (n16 units of 16 bytes each) to up to three places
+struct CopyParts {
+    struct Part {
+        const void* src;
+        void* dst[3];
+        long long n16;
+    } part[32];
+    int n;
+};
+cudaError_t launch_copy_parts(const CopyParts& C, int sms, cudaStream_t st);
 cudaError_t launch_set_field(const Params& P, int comp, const float* dense, float* dst, double scale,
                              cudaStream_t st);
 cudaError_t launch_prime(const Params& P, cudaStream_t st);

@@ -138,3 +138,25 @@ def test_batches_in_place_and_staged(sizes, count):
     for w, a, b in zip(ws, *runs):
         assert a.level == 41
         _same(a, b, w, 41)
+
+
+@pytest.mark.parametrize("cap,max_probes,mu", [(71, 1, (1.0, 1.0)), (71, 3, (1.0, 2.0)), (72, 2, (1.0, 2.0))])
+def test_adjoint_checkpoints_leave_the_forward_state(cap, max_probes, mu):
+    """The adjoint's checkpoints hold every part, a series of odd length among
+    them, and a restore leaves all buffers as a run without it does."""
+    from paper_2305_13419_gb300 import twofluid as tf
+    w = _workload((40, 9, 11), (C, P, C), 0, 1.0, mu)
+    w.probes = w.probes[:1]
+    runs = []
+    for adjoint in (True, False):
+        g = tf.Grid.from_workload(w, series_capacity=cap, max_probes=max_probes)
+        if adjoint:
+            g.adjoint(50, 0, 0, segment=9)
+        else:
+            g.step(50)
+        g.step(12)   # the state is also good to go on from, in place and staged
+        g.set_wait_limit(1 << 21)
+        g.step(7)
+        g.sync()
+        runs.append(g)
+    _same(runs[0], runs[1], w, 50)
