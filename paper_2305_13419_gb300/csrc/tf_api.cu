@@ -1479,6 +1479,10 @@ tf_status tf_read_probe_dft(tf_handle h, int id, double* re, double* im) {
     const int nf = h->R.nfreq[id];
     // both sums in one copy: they lie a fixed distance apart
     double both[2][TF_MAX_FREQS];
+    if (nf == 0) {
+        TF_CUDA(cudaStreamSynchronize(h->stream));
+        return TF_OK;
+    }
     TF_CUDA(cudaMemcpy2DAsync(both, sizeof(both[0]), h->R.re + id * TF_MAX_FREQS,
                               (size_t)((const char*)h->R.im - (const char*)h->R.re), sizeof(double) * nf, 2,
                               cudaMemcpyDeviceToHost, h->stream));

@@ -160,3 +160,12 @@ def test_adjoint_checkpoints_leave_the_forward_state(cap, max_probes, mu):
         g.sync()
         runs.append(g)
     _same(runs[0], runs[1], w, 50)
+
+
+def test_probe_without_frequencies_reads_an_empty_spectrum():
+    w = _workload((20, 9, 11), (P, P, C), 0, 1.0, (1.0, 1.0))
+    w.probes = [W.Probe(comp=0, p=(3, 4, 5), freqs=np.zeros(0), series=9), w.probes[1]]
+    g = _grid(w, False)
+    g.step(9)
+    assert g.probe_dft(0).size == 0 and g.probe_series(0, 9).size == 9
+    assert g.probe_dft(1).size > 0
