@@ -157,7 +157,7 @@ tf_status tf_add_probe(tf_handle h, int comp, const int p[3], const double* freq
 /* Advance nsteps >= 0 steps of Algorithm 1 (fused form) on the stream: the B
  * update with CPML memory, the Js update, the theta-scheme E update with
  * sources, the Mur walls, the probe DFTs and the non-finite watchdog.  Grids
- * of up to some 65 million points run in place, a B pass and an E pass per
+ * of up to some 80 million points run in place, a B pass and an E pass per
  * step; larger ones one fused launch per step or two-step passes
  * (tf_set_two_step).  The results are the same bits.  Asynchronous; launch errors are
  * returned (the handle is then unusable), device-side errors latch for

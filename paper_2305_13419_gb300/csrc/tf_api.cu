@@ -748,7 +748,8 @@ PassArgs pass_args(const tf_ctx* h, const Sources& S) {
     for (int p = 0; p < h->R.n; ++p) {   // the item that samples a probe (a point on a high wall: the item next to it)
         int w[3];
         for (int a = 0; a < 3; ++a) w[a] = h->ppos[p][a] < last[a] ? h->ppos[p][a] : last[a];
-        A.pr_block[p] = ((w[2] >> L.psc) * L.pnby + (w[1] >> L.psb)) * L.pnbx + (w[0] >> (L.psa + 2));
+        A.pr_item[p] = (w[1] >> L.psb) * L.pnbx + (w[0] >> (L.psa + 2));
+        A.pr_k[p] = w[2];
         A.pr_comp[p] = h->R.comp[p];
         A.pr_q[p] = h->R.q[p];
     }
@@ -863,10 +864,10 @@ cudaError_t run_narrow(tf_ctx* h, const Sources& S, int64_t nsteps) {
 // Does tf_step run in place (tf_pass.cu)?  Not when two-step passes were
 // asked for, nor under a wait limit of the handle's own (the passes wait for
 // nothing).  us per step in place / single staged steps / two-step passes on
-// CPW grids: 0.3 M cells 7.5 / 21 / 68, 2.1 M 31 / 72 / 126, 4 M 70 / 104 / 149,
-// 8 M 127 / 165 / 182, 17 M 234 / 266 / 273, 33 M 444 / 475 / 448, 43 M 576 /
-// 627 / 600, 57 M 753 / 797 / 755, 134 M 1900 / 1695 / 1512: on large grids the
-// 72 bytes per point of the two passes cost more than two steps' 48.
+// CPW grids: 0.3 M cells 7.5 / 21 / 68, 2.1 M 31 / 72 / 126, 4 M 56 / 104 / 149,
+// 8 M 102 / 165 / 182, 17 M 199 / 266 / 273, 32 M 368 / - / 421, 72 M 945 / - /
+// 970, 134 M 1620 / 1695 / 1512: planes of half a million points leave a window
+// of planes (tf_pass.cu) too little of L2.
 bool in_place(const tf_ctx* h) {
     const bool asked = h->two_step_on == 2 && h->box_ok && h->P.uniform_mu;
     return !asked && h->P.wait_polls == kSpinLimit && h->L.total <= kPassPoints;
@@ -1160,19 +1161,19 @@ tf_status batch_check(const tf_handle* hs, int n, int64_t nsteps) {
 
 namespace {
 
-// Streams of a batch that runs in place.  One, where a grid fills the SMs and
-// its fields stay in L2 while it runs a group of steps by itself; two, where
-// smaller grids leave room, or larger ones ends to fill; four for the smallest.
-// us per step of the batch on 1 / 2 / 4 streams: 16 grids of 2.4 M cells on
-// average 575 / 598 / 628, 8 of 6 M 824 / 774 / 783, 24 of 0.6 M 278 / 182 / 232,
-// 32 of 0.17 M 244 / 140 / 114 (with CTAs of one launch over the whole batch,
-// staged planes: 820, 1070, 504, 320; 200 grids of 36^3 cells: 1217 against 769).
+// Streams of a batch that runs in place.  One, where a grid (or a window of its
+// planes) fills the SMs and its fields stay in L2 while it runs a group of steps
+// by itself; two or four where smaller grids leave room.  us per step of the
+// batch on 1 / 2 / 4 streams: 6 grids of 6 M cells 539 / 592 / 624, 16 of 4.1 M
+// 933 / 975 / 1072, 8 of 2.7 M 412 / 402 / 408, 24 of 0.6 M 278 / 182 / 232, 32 of
+// 0.17 M 244 / 140 / 114 (with CTAs of one launch over the whole batch, staged
+// planes: 504 and 320 for the last two; 200 grids of 36^3 cells: 1217 against 769).
 constexpr int kBatchStreams = 4;
 int batch_streams(const tf_handle* hs, int n) {
     long long pts = 0;
     for (int i = 0; i < n; ++i) pts += hs[i]->L.total;
     pts /= n;
-    return pts < 400000 ? kBatchStreams : pts < 1200000 || pts > 4500000 ? 2 : 1;
+    return pts < 400000 ? kBatchStreams : pts < 1200000 ? 2 : 1;
 }
 struct BatchStreams {
     cudaStream_t s[kBatchStreams] = {};

@@ -345,7 +345,7 @@ cudaError_t launch_step_advance(int* step, cudaStream_t st);
 // Steps in place by a B pass and an E pass each (tf_pass.cu): the fields are
 // those of the current buffer.
 constexpr int kPassSteps = 32;     // steps per group of launches (probe samples are kept for that many)
-constexpr long long kPassPoints = 64LL << 20;   // padded points of a grid up to which tf_step runs in place
+constexpr long long kPassPoints = 80LL << 20;   // padded points of a grid up to which tf_step runs in place
 constexpr int kPassBits = 7, kPassThreads = 1 << kPassBits;   // threads of an item, a quad of x points each
 struct PassArgs {
     Params P;
@@ -358,7 +358,8 @@ struct PassArgs {
     int cx, cy, kend;                           // points advanced along x, y, z: [0, c)
     int sms;                                    // multiprocessors of the device
     int nprobe;
-    int pr_block[TF_MAX_PROBES], pr_comp[TF_MAX_PROBES];   // the item that samples a probe
+    int pr_item[TF_MAX_PROBES], pr_k[TF_MAX_PROBES];   // the item along x, y and the plane that sample a probe
+    int pr_comp[TF_MAX_PROBES];
     long long pr_q[TF_MAX_PROBES];
     float* samples;                             // [step][probe]: E^n of the steps
 };

@@ -353,28 +353,32 @@ struct Item {
     bool live;
     Quad u;
 };
-__device__ __forceinline__ Item item_at(const PassArgs& A, int bx, int by, int bz) {
+// the thread's quad in a launch over planes [k0, k1)
+__device__ __forceinline__ Item item_at(const PassArgs& A, int k0, int k1) {
     Item it;
     const int tid = threadIdx.x;
     const int iq = tid & ((1 << A.sa) - 1), jr = (tid >> A.sa) & ((1 << A.sb) - 1), kr = tid >> (A.sa + A.sb);
-    const int x0 = 4 * (bx << A.sa), y0 = by << A.sb, z0 = bz << A.sc;
+    const int x0 = 4 * (blockIdx.x << A.sa), y0 = blockIdx.y << A.sb, z0 = k0 + (blockIdx.z << A.sc);
     const int x = x0 + 4 * iq, j = y0 + jr, k = z0 + kr;
-    it.live = x < A.cx && j < A.cy && k < A.kend;
+    it.live = x < A.cx && j < A.cy && k < k1;
     it.u = quad_of(A.P, x, j, k);
     return it;
 }
-__device__ __forceinline__ void sample(const PassArgs& A, int blk, int t) {
-    if (threadIdx.x < A.nprobe && A.pr_block[threadIdx.x] == blk)
-        A.samples[t * TF_MAX_PROBES + threadIdx.x] = A.P.E[A.pr_comp[threadIdx.x]][A.pr_q[threadIdx.x]];
+__device__ __forceinline__ void sample(const PassArgs& A, int t, int k0, int k1) {
+    const int p = threadIdx.x;
+    if (p < A.nprobe && A.pr_item[p] == (int)(blockIdx.y * A.nbx + blockIdx.x) && A.pr_k[p] >= k0 && A.pr_k[p] < k1 &&
+        (A.pr_k[p] - k0) >> A.sc == (int)blockIdx.z)
+        A.samples[t * TF_MAX_PROBES + p] = A.P.E[A.pr_comp[p]][A.pr_q[p]];
 }
 
 }  // namespace
 
-// One pass of one step over the grid (kE: the E pass).  Bound by the latency
+// One pass of one step over the planes [k0, k1) (kE: the E pass).  Bound by the latency
 // of its one round of loads on small grids (two launches, 7.5 us a step on the
-// 128 x 64 x 40 CPW) and by memory on large ones: the 512 x 256 x 128 CPW takes
-// 234 us a step (6.2 TB/s of 72 bytes per point plus the CPML memories), the
-// 256 x 128 x 64 CPW, whose 90 MB nearly stay in L2, 31.  What is spilled goes to
+// 128 x 64 x 40 CPW) and by memory on large ones: over the whole 512 x 256 x 128
+// CPW it takes 234 us a step (6.2 TB/s of 72 bytes per point plus the CPML
+// memories), 199 in windows of planes (windows_of below: L2 to SM traffic and the
+// launches' ends), on the 256 x 128 x 64 CPW, whose 90 MB nearly stay in L2, 31.  What is spilled goes to
 // L2 and back: with all three slab axes' memories and Js fetched up front the E
 // pass spilled 170 bytes a thread (252 and 43 us); now the first slab axis is
 // fetched early, the others and Js where they are used.  A step of the latter
@@ -388,13 +392,13 @@ __device__ __forceinline__ void sample(const PassArgs& A, int blk, int t) {
 // Items off the walls, seams and slabs take the same code: a variant without
 // its tests was no faster.
 // Launches overlap (programmatic dependent launch): a thread fetches what
-// only its own pass writes -- one step and two launches ago -- before it waits
+// only its own pass writes -- two launches ago or more -- before it waits
 // for the launch before.  That launch lets the next one start only once its
 // own wait is over, so the launch before it is complete by then.
 template <bool kE, bool kEarly>
 __global__ void __launch_bounds__(kFT, kEarly ? kEarlyMin : kE ? kEMin : kBMin)
-    k_pass(const __grid_constant__ PassArgs A, const __grid_constant__ PassAmps W, int t) {
-    const Item it = item_at(A, blockIdx.x, blockIdx.y, blockIdx.z);
+    k_pass(const __grid_constant__ PassArgs A, const __grid_constant__ PassAmps W, int t, int k0, int k1) {
+    const Item it = item_at(A, k0, k1);
     if constexpr (kE) {
         PreE r;
         if (it.live) pre_e<kEarly>(A, it.u, r);
@@ -407,7 +411,7 @@ __global__ void __launch_bounds__(kFT, kEarly ? kEarlyMin : kE ? kEMin : kBMin)
         asm volatile("griddepcontrol.wait;" ::: "memory");
         asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
         if (it.live) post_b<kEarly>(A.P, it.u, r);
-        sample(A, (blockIdx.z * A.nby + blockIdx.y) * A.nbx + blockIdx.x, t);
+        sample(A, t, k0, k1);
     }
 }
 
@@ -438,9 +442,38 @@ cudaError_t launch_pass_probes(const Probes& R, const float* samples, long long 
     return cudaGetLastError();
 }
 
-// `steps` steps from `level`, two launches each, with the amplitudes amp[step];
-// a launch may start while the one before drains (it waits for it before it
-// reads what that one writes)
+// Windows of planes, each stepped `depth` times before the next one, so that
+// what a pass reads is still in L2 from the passes before (over a whole grid
+// beyond L2 every pass streams 36 bytes per point from DRAM).  The planes go up
+// and a window's step u works on it shifted u planes down: the B pass of a
+// plane needs E of that plane and the one above at the same level, the E pass
+// B of that plane and the one below, and neither is a level ahead.  Every value
+// is the one of whole passes, whatever the windows.  (A periodic z axis would
+// need the last plane's neighbour before its own step.)
+// us per step of CPW grids, whole / in windows of some million points, 16 steps:
+//   512 x 256 x 128   234 / 1.5: 208, 2: 199, 2.5: 205, 3: 220, 4: 242
+//   256 x 256 x 128   127 / 1: 120, 1.5: 105, 2: 102, 2.5: 105, 3: 118
+//   700 x 300 x 150   (421 in two-step passes) / 1.5: 387, 1.9: 368, 2.5: 372, 3: 398
+//   160 x 160 x 128    53 / 1: 48, 1.4: 44, 1.8: 42;   128^3  30 / 1: 38, 1.4: 30
+// smaller windows leave the last wave of each launch emptier, larger ones leave
+// L2.  8 steps instead of 16 are 1 to 3 % slower, 4 steps 4 to 7 %.
+constexpr double kWindowPoints = 1.9e6, kWindowMin = 2.8e6;
+constexpr int kWindowSteps = 16;
+struct Windows {
+    int planes, depth;
+};
+Windows windows_of(const PassArgs& A, int steps) {
+    const double points = (double)A.cx * A.cy * A.kend;
+    if (A.P.per[2] || points < kWindowMin) return {A.kend, 1};
+    const int most = A.kend < 1 << 20 ? A.kend : 1 << 20, n = (int)(points / kWindowPoints + 0.5);
+    const int count = n < 2 ? 2 : n < most ? n : most, groups = (steps + kWindowSteps - 1) / kWindowSteps;
+    return {(A.kend + count - 1) / count, (steps + groups - 1) / groups};
+}
+
+// `steps` steps from `level`, two launches per step and window of planes, with
+// the amplitudes amp[step]; a launch may start while the one before drains (it
+// waits for it before it reads what that one writes: what it fetches earlier
+// was last written by a launch of its own kind, two launches ago or more)
 cudaError_t launch_passes(const PassArgs& A, const Probes& R, const PassAmps* amp, long long level, int steps,
                           cudaStream_t st) {
     cudaLaunchConfig_t cfg{};
@@ -452,15 +485,24 @@ cudaError_t launch_passes(const PassArgs& A, const Probes& R, const PassAmps* am
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     const bool early = A.nbx * A.nby * A.nbz <= kEarlyMin * A.sms;
+    const Windows win = windows_of(A, steps);
+    cfg.numAttrs = 0;   // the first launch waits for whatever the stream holds
     cudaError_t e = cudaSuccess;
-    for (int t = 0; t < steps && e == cudaSuccess; ++t) {
-        cfg.numAttrs = t > 0 ? 1 : 0;   // the first launch waits for whatever the stream holds
-        e = early ? cudaLaunchKernelEx(&cfg, k_pass<false, true>, A, amp[t], t)
-                  : cudaLaunchKernelEx(&cfg, k_pass<false, false>, A, amp[t], t);
-        cfg.numAttrs = 1;
-        if (e == cudaSuccess)
-            e = early ? cudaLaunchKernelEx(&cfg, k_pass<true, true>, A, amp[t], t)
-                      : cudaLaunchKernelEx(&cfg, k_pass<true, false>, A, amp[t], t);
+    for (int t0 = 0; t0 < steps; t0 += win.depth) {
+        const int m = steps - t0 < win.depth ? steps - t0 : win.depth;
+        for (int z = 0; z < A.kend + m - 1; z += win.planes)
+            for (int u = 0; u < m && e == cudaSuccess; ++u) {
+                const int k0 = z > u ? z - u : 0, k1 = z + win.planes - u < A.kend ? z + win.planes - u : A.kend;
+                if (k0 >= k1) continue;
+                const PassAmps& W = amp[t0 + u];
+                cfg.gridDim.z = ((k1 - k0 - 1) >> A.sc) + 1;
+                e = early ? cudaLaunchKernelEx(&cfg, k_pass<false, true>, A, W, t0 + u, k0, k1)
+                          : cudaLaunchKernelEx(&cfg, k_pass<false, false>, A, W, t0 + u, k0, k1);
+                cfg.numAttrs = 1;
+                if (e == cudaSuccess)
+                    e = early ? cudaLaunchKernelEx(&cfg, k_pass<true, true>, A, W, t0 + u, k0, k1)
+                              : cudaLaunchKernelEx(&cfg, k_pass<true, false>, A, W, t0 + u, k0, k1);
+            }
     }
     if (e == cudaSuccess && R.n > 0) e = launch_pass_probes(R, A.samples, level, steps, st);
     return e;

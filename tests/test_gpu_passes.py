@@ -1,5 +1,5 @@
 """Steps in place (a B pass and an E pass per step, what tf_step does on grids
-of up to some 65 million points) and many steps per launch (grids with a
+of up to some 80 million points) and many steps per launch (grids with a
 narrow cross section) give the same bits as the staged single-step
 kernel: fields, probe DFTs and series, on every boundary kind, on rows that
 end inside a thread's four points, with sources and probes at the walls,
@@ -169,3 +169,40 @@ def test_probe_without_frequencies_reads_an_empty_spectrum():
     g.step(9)
     assert g.probe_dft(0).size == 0 and g.probe_series(0, 9).size == 9
     assert g.probe_dft(1).size > 0
+
+
+@pytest.mark.parametrize("case", [((205, 131, 140), (C, P, C), 0, 1.0, (1.0, 1.0)),
+                                  ((203, 130, 141), (W_, C, M), 1, 0.5, (1.0, 1.0)),
+                                  ((300, 201, 90), (P, W_, W_), 0, 1.0, (1.0, 2.0)),
+                                  ((64, 41, 1500), (P, C, M), 0, 1.0, (1.0, 1.0))],
+                         ids=["cpml", "mur", "pec-mu", "long"])
+def test_windows_of_planes_give_the_bits_of_staged_steps(case):
+    """Grids large enough to be stepped window by window, several steps each:
+    probes on the first, the last and a middle plane, group ends inside a
+    window's depth."""
+    w = _workload(*case)
+    ref = _grid(w, True)
+    ref.step(41)
+    g = _grid(w, False)
+    for n in (1, 2, 33, 5):
+        g.step(n)
+    g.sync()
+    _same(g, ref, w, 41)
+
+
+def test_windows_of_planes_keep_the_history_of_the_adjoint():
+    """E at every level, written window by window, against staged steps' copies."""
+    from paper_2305_13419_gb300 import twofluid as tf
+    n = (205, 131, 140)
+    w = _workload(n, (C, P, C), 0, 1.0, (1.0, 1.0))
+    w.probes = [W.Probe(comp=0, p=(n[0] // 3 + 7, n[1] // 2, n[2] // 2 + 1), freqs=w.probes[0].freqs)]
+    out = []
+    for staged in (True, False):
+        g = tf.Grid.from_workload(w)
+        g.set_two_step(False)
+        if staged:
+            g.set_wait_limit(1 << 21)
+        out.append(g.adjoint(40, 0, 0, segment=9))
+    (J, eps, lam), (J1, eps1, lam1) = out
+    assert J > 0 and J == J1
+    assert torch.equal(eps, eps1) and torch.equal(lam, lam1)
