@@ -479,9 +479,8 @@ def run_adjoint(args):
         from paper_2305_13419_gb300 import autotune
         tuning = autotune.tune_grid(g, steps=args.autotune_steps)
     g.step(20)
-    _, tot = g.step_timed(200, with_total=True)
+    plain = g.time_steps(200) / 200
     g.sync()
-    plain = tot / 200
     g.close()
     del g
     g = tf.Grid.from_workload(w)
@@ -504,9 +503,8 @@ def run_adjoint(args):
 
 def run_batch(args, plain_gcells, plain_workload="cpw-512x256x128"):
     """The batched workload: 64 CPW variants with axes from {96, 128, 160}.
-    Headline: tf_batch_run, one launch per step over all 64 grids (one work
-    list over all grids' items), 64 steps per CUDA graph, timed with CUDA
-    events on its stream; beside it tf_batch_step (per-grid launches spread
+    Headline: tf_batch_run (grid by grid in place, groups of 32 steps), timed
+    with CUDA events around the call; beside it tf_batch_step (per-grid launches spread
     over 8 streams)."""
     import time
     import torch
@@ -516,7 +514,7 @@ def run_batch(args, plain_gcells, plain_workload="cpw-512x256x128"):
     cells = sum(w.ncells for w in ws)
     out = {"grids": len(ws), "cells": cells, "steps": args.batch_steps, "sizes": [96, 128, 160]}
     grids = [tf.Grid.from_workload(w) for w in ws]
-    # algorithmic bytes of one batched launch: every grid's one-pass bytes
+    # algorithmic bytes of one step of all grids: every grid's one-pass bytes
     ab = sum(algorithmic_bytes(w, g.N)["step"] for w, g in zip(ws, grids))
     tf.batch_run(grids, 10)
     torch.cuda.synchronize()
@@ -534,15 +532,14 @@ def run_batch(args, plain_gcells, plain_workload="cpw-512x256x128"):
     torch.cuda.empty_cache()
     peak, peak_kind = hbm_peak()
     mps = ms / args.batch_steps
-    out["one_launch"] = {"ms_per_step": mps,
-                         "gcell_updates_per_s": cells * args.batch_steps / (ms * 1e-3) / 1e9,
-                         "timing": "CUDA events on the batch's stream around tf_batch_run (includes its set-up "
-                                   "uploads and graph capture)",
-                         "roofline": {"bound": "hbm", "kernel": "k_step_t<batch>", "algorithmic_bytes": ab,
-                                      "achieved": ab / (mps * 1e-3) / 1e9, "peak": peak, "unit": "GB/s",
-                                      "frac": ab / (mps * 1e-3) / 1e9 / peak,
-                                      "traffic": ncu_traffic("k_step_batch", "batch-64-cpw"),
-                                      "peak_source": peak_kind}}
+    out["batch_run"] = {"ms_per_step": mps,
+                        "gcell_updates_per_s": cells * args.batch_steps / (ms * 1e-3) / 1e9,
+                        "timing": "CUDA events on the first grid's stream around tf_batch_run, which returns when "
+                                  "every grid is done",
+                        "roofline": {"bound": "hbm", "kernel": "k_pass", "algorithmic_bytes": ab,
+                                     "achieved": ab / (mps * 1e-3) / 1e9, "peak": peak, "unit": "GB/s",
+                                     "frac": ab / (mps * 1e-3) / 1e9 / peak, "traffic": None,
+                                     "peak_source": peak_kind}}
     streams = [torch.cuda.Stream() for _ in range(8)]
     grids = [tf.Grid.from_workload(w, stream=streams[i % 8]) for i, w in enumerate(ws)]
     for gg in grids:   # single steps, as in the batched launch (the autotuner's choice on grids this small)
@@ -561,7 +558,7 @@ def run_batch(args, plain_gcells, plain_workload="cpw-512x256x128"):
     out["streams8"] = {"ms_per_step": ms / args.batch_steps,
                        "gcell_updates_per_s": cells * args.batch_steps / (ms * 1e-3) / 1e9,
                        "timing": "host wall clock around the enqueue of all steps, device synchronised on both sides"}
-    out["gcell_updates_per_s"] = out["one_launch"]["gcell_updates_per_s"]
+    out["gcell_updates_per_s"] = out["batch_run"]["gcell_updates_per_s"]
     out["vs_plain_step"] = out["gcell_updates_per_s"] / plain_gcells
     out["plain_step"] = {"workload": plain_workload, "gcell_updates_per_s": plain_gcells}
     return out
@@ -636,10 +633,10 @@ def run_batch_overhead(args):
 
 
 def run_config(w, steps, warmup=5, two_step=True, autotune_steps=0):
-    """GPU throughput of the plain step on one workload: the whole run and
-    the step kernel's own launches timed with CUDA events on the handle's
-    stream over the same launches; the kernel's algorithmic bytes over its
-    mean launch time give the roofline fraction."""
+    """GPU throughput of tf_step on one workload, timed whole with CUDA events
+    on the handle's stream; beside it the staged kernels' own launches
+    (tf_step_timed, which grids that tf_step runs in place take as well): their
+    algorithmic bytes over the mean launch time give the roofline object."""
     import torch
     from paper_2305_13419_gb300 import twofluid as tf
     g = tf.Grid.from_workload(w)
@@ -652,7 +649,9 @@ def run_config(w, steps, warmup=5, two_step=True, autotune_steps=0):
     g.step(warmup)
     g.sync()
     torch.cuda.synchronize()
-    kt, ms = g.step_timed(steps, with_total=True)
+    ms = g.time_steps(steps)
+    g.sync()
+    kt, _ = g.step_timed(max(20, steps // 10), with_total=True)
     g.sync()
     _, roof = roofline_of(w, g, kt, planes=tuning["best"] if tuning and tuning["best"] else 24,
                           item_planes=tuning["item_planes"] if tuning else 8)

@@ -11,8 +11,8 @@ how the work is cut), so the tuner only times.  What it chooses:
     (tf_set_item_planes): long items on large grids, short ones where a
     grid has few items per CTA.
 
-A batch (tf_batch_run) needs no split to tune: its grids' work items form
-one list that the launch's CTAs share through one counter.
+A batch (tf_batch_run) needs no split to tune: its grids run in place one
+after the other, or their work items form one list.
 
 The tile shape (32 x 16 columns, 8-plane single-step items) is fixed when the
 kernels are compiled; the shapes measured against it are listed in the
@@ -28,8 +28,13 @@ ITEM_PLANES_CANDIDATES = (8, 16)       # planes per single-step work item
 
 
 def _time_steps(grid, steps: int) -> float:
-    """ms per step of `steps` steps of `grid`, CUDA events on its stream."""
-    _, total = grid.step_timed(steps, with_total=True)
+    """ms per step of `steps` steps of `grid`, CUDA events on its stream: what
+    tf_step takes (grids that it steps in place run there with two-step passes
+    off), or the staged kernels where only those can be timed."""
+    if hasattr(grid, "time_steps"):
+        total = grid.time_steps(steps)
+    else:
+        _, total = grid.step_timed(steps, with_total=True)
     grid.sync()
     return total / steps
 

@@ -449,6 +449,18 @@ class Grid:
     def sync(self):
         tf_sync(self.h)
 
+    def time_steps(self, nsteps: int) -> float:
+        """Advances nsteps by tf_step and returns the ms they took on the
+        grid's stream (CUDA events around the call)."""
+        import torch
+        st = self.stream
+        e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        e0.record(st)
+        self.step(nsteps)
+        e1.record(st)
+        e1.synchronize()
+        return e0.elapsed_time(e1)
+
     def step_timed(self, nsteps: int, with_total: bool = False):
         """Advance like step(); returns {kernel: (mean ms per launch, launches)}
         for the single-step kernel ("step") and the two-step kernel ("step2")
