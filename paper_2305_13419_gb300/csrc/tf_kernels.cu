@@ -186,23 +186,62 @@ __device__ __forceinline__ float read_point(const Params& P, int c, int primed, 
     }
 }
 
+// four points of a row of B_c (32 apart, from i0): every load that all points
+// need before the first use, at positions kept inside the row
+template <int kC>
+__device__ __forceinline__ void read_b_row(const Params& P, int primed, int i0, int j, int k, float sh, float sl, float v[4]) {
+    constexpr int a1 = kC == 0 ? 1 : 0, a2 = kC == 2 ? 1 : 2;
+    const float *e1 = P.E[3 - kC - a1], *e2 = P.E[3 - kC - a2];
+    const int row = (int)lin(P, 0, j, k);
+    const int rows[3] = {row, (int)lin(P, 0, nxt(P, 1, j), k), (int)lin(P, 0, j, nxt(P, 2, k))};
+    auto past = [&](int a, int x) { return a == 0 ? row + nxt(P, 0, x) : rows[a] + x; };
+    float d1[4], d2[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int x = min(i0 + 32 * u, P.N[0] - 1);
+        v[u] = P.B[kC][row + x];
+        d1[u] = e1[past(a1, x)] - e1[row + x];
+        d2[u] = e2[past(a2, x)] - e2[row + x];
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int p[3] = {min(i0 + 32 * u, P.N[0] - 1), j, k}, q = row + p[0];
+        if (primed && upd_B(P, kC, p)) {   // curl_E_peek of the loaded differences
+            float t1 = P.r[a1] * d1[u], t2 = P.r[a2] * d2[u];
+            if (P.psiB[kC][a1] && in_slab(P, a1, p[a1]))
+                t1 += P.pbB[a1][p[a1]] * P.psiB[kC][a1][q] + P.pcB[a1][p[a1]] * d1[u];
+            if (P.psiB[kC][a2] && in_slab(P, a2, p[a2]))
+                t2 += P.pbB[a2][p[a2]] * P.psiB[kC][a2][q] + P.pcB[a2][p[a2]] * d2[u];
+            v[u] -= 0.5f * (curl_sign(kC, a1) * t1 + curl_sign(kC, a2) * t2);
+        }
+        v[u] = scaled(v[u], sh, sl);
+    }
+}
+
 // Read-back.  Bound by memory: a warp takes 128 points of a row, four loads of
-// each array in flight per thread.  (It was one thread per point with 64-bit
-// divisions and three FP64 operations a point, 2 FP64 lanes per cycle and SM:
-// nine fields of the 1024 x 512 x 256 CPW took 9.3 ms.)  kRows = false: rows
-// shorter than a warp, points in sequence.
-template <int kKind, bool kRows>
-__global__ void __launch_bounds__(256) k_read_field(Params P, int c, int primed, const float4* tilemat, int ntx,
+// each array in flight per thread, the component a constant.  Nine fields of the
+// 1024 x 512 x 256 CPW take 2.6 ms: E 0.18 each (5.9 TB/s), Js 0.20, B 0.46 to
+// 0.51 (four arrays' worth at 4.4 TB/s), whose 0.83 were bound by instructions
+// and by loads one after the other while the component was an argument and each
+// point formed its curl by itself.  (9.3 ms with one thread per point, 64-bit
+// divisions and three FP64 operations a point, 2 FP64 lanes per cycle and SM.)
+// kRows = false: rows shorter than a warp, points in sequence.
+template <int kKind, int kC, bool kRows>
+__global__ void __launch_bounds__(256) k_read_field(Params P, int primed, const float4* tilemat, int ntx,
                                                     float* dense, float sh, float sl) {
     if constexpr (kRows) {
         const int j = blockIdx.y * 8 + threadIdx.y, k = blockIdx.z, i0 = blockIdx.x * 128 + threadIdx.x;
         if (j >= P.N[1]) return;
         float* const out = dense + ((long long)k * P.N[1] + j) * P.N[0];
         float v[4];
+        if constexpr (kKind == 1) {
+            read_b_row<kC>(P, primed, i0, j, k, sh, sl, v);
+        } else {
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int p[3] = {i0 + 32 * u, j, k};
-            if (p[0] < P.N[0]) v[u] = read_point<kKind>(P, c, primed, tilemat, ntx, p, sh, sl);
+            for (int u = 0; u < 4; ++u) {
+                const int p[3] = {i0 + 32 * u, j, k};
+                if (p[0] < P.N[0]) v[u] = read_point<kKind>(P, kC, primed, tilemat, ntx, p, sh, sl);
+            }
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u)
@@ -210,7 +249,7 @@ __global__ void __launch_bounds__(256) k_read_field(Params P, int c, int primed,
     } else {
         const unsigned t = blockIdx.x * 256u + threadIdx.x, row = t / (unsigned)P.N[0];
         const int p[3] = {(int)(t - row * (unsigned)P.N[0]), (int)(row % (unsigned)P.N[1]), (int)(row / (unsigned)P.N[1])};
-        if (p[2] < P.N[2]) dense[t] = read_point<kKind>(P, c, primed, tilemat, ntx, p, sh, sl);
+        if (p[2] < P.N[2]) dense[t] = read_point<kKind>(P, kC, primed, tilemat, ntx, p, sh, sl);
     }
 }
 
@@ -274,27 +313,37 @@ cudaError_t launch_prime(const Params& P, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-template <int kKind>
-static void read_kernel(const Params& P, int c, int primed, const float4* tilemat, int ntx, float* dense, float sh,
-                        float sl, cudaStream_t st) {
+template <int kKind, int kC>
+static void read_kernel(const Params& P, int primed, const float4* tilemat, int ntx, float* dense, float sh, float sl,
+                        cudaStream_t st) {
     if (P.N[0] >= 32 && P.N[1] <= 8 * 65535 && P.N[2] <= 65535) {   // (blockIdx.y and z end there)
-        k_read_field<kKind, true><<<dim3((P.N[0] + 127) / 128, (P.N[1] + 7) / 8, P.N[2]), dim3(32, 8), 0, st>>>(
-            P, c, primed, tilemat, ntx, dense, sh, sl);
+        k_read_field<kKind, kC, true><<<dim3((P.N[0] + 127) / 128, (P.N[1] + 7) / 8, P.N[2]), dim3(32, 8), 0, st>>>(
+            P, primed, tilemat, ntx, dense, sh, sl);
     } else {
         const long long tot = (long long)P.N[0] * P.N[1] * P.N[2];
-        k_read_field<kKind, false><<<blocks_for(tot, 256), 256, 0, st>>>(P, c, primed, tilemat, ntx, dense, sh, sl);
+        k_read_field<kKind, kC, false><<<blocks_for(tot, 256), 256, 0, st>>>(P, primed, tilemat, ntx, dense, sh, sl);
     }
+}
+template <int kKind>
+static void read_kernel_of(const Params& P, int c, int primed, const float4* tilemat, int ntx, float* dense, float sh,
+                           float sl, cudaStream_t st) {
+    if (c == 0)
+        read_kernel<kKind, 0>(P, primed, tilemat, ntx, dense, sh, sl, st);
+    else if (c == 1)
+        read_kernel<kKind, 1>(P, primed, tilemat, ntx, dense, sh, sl, st);
+    else
+        read_kernel<kKind, 2>(P, primed, tilemat, ntx, dense, sh, sl, st);
 }
 
 cudaError_t launch_read_field(const Params& P, int comp, int primed, const float4* tilemat, int ntx, float* dense,
                               double scale, cudaStream_t st) {
     const float sh = (float)scale, sl = (float)(scale - (double)sh);
     if (comp < 3)
-        read_kernel<0>(P, comp, primed, tilemat, ntx, dense, sh, sl, st);
+        read_kernel_of<0>(P, comp, primed, tilemat, ntx, dense, sh, sl, st);
     else if (comp < 6)
-        read_kernel<1>(P, comp - 3, primed, tilemat, ntx, dense, sh, sl, st);
+        read_kernel_of<1>(P, comp - 3, primed, tilemat, ntx, dense, sh, sl, st);
     else
-        read_kernel<2>(P, comp - 6, primed, tilemat, ntx, dense, sh, sl, st);
+        read_kernel_of<2>(P, comp - 6, primed, tilemat, ntx, dense, sh, sl, st);
     return cudaGetLastError();
 }
 
