@@ -809,7 +809,7 @@ cudaError_t run_narrow(tf_ctx* h, const Sources& S, int64_t nsteps) {
     const int most = (A.window - 1) / 2, least = A.window / 4 < kPassSteps ? A.window / 4 : kPassSteps;
     const int dft = (h->R.n * TF_MAX_FREQS + kNarrowThreads / 32 - 1) / (kNarrowThreads / 32);
     int depth = most < kPassSteps ? most : kPassSteps;
-    while (depth > least && (h->L.N[2] + A.window - 2 * depth - 1) / (A.window - 2 * depth) + dft > h->sms) --depth;
+    while (depth > least && narrow_blocks(h->P, A.window - 2 * depth) + dft > h->sms) --depth;
     // psi_E has one array per component: the third psi_B buffer, which only
     // two-step passes use (a narrow grid has no box for them), is its other one
     float* pe[2][2];

@@ -392,6 +392,11 @@ struct NarrowArgs {
     int steps_before;
     int chained;                   // the launch before in the stream is one of these
 };
+// windows of a launch: a Mur wall is not counted, it goes with the plane next to it
+inline int narrow_blocks(const Params& P, int own) {
+    const int planes = P.bc[2] == TF_BC_MUR ? P.n[2] : P.N[2];
+    return (planes + own - 1) / own;
+}
 cudaError_t launch_narrow(const NarrowArgs& A, const Probes& R, cudaStream_t st);
 cudaError_t launch_face_imu(const Params& P, float* const w[3], cudaStream_t st);
 

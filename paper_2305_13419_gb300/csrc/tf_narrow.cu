@@ -6,6 +6,8 @@
 // one down (Bt at plane k reads E at k and k + 1, E reads Bt at k and k - 1),
 // so what the window's ends lack spoils one plane per step and the owned
 // planes come out right after all of them, without a word between CTAs.
+// (A Mur wall takes up the new E of the plane next to it and is right only as
+// long as that plane is: the CTA that owns that plane owns the wall as well.)
 // A thread keeps four x-adjacent points -- E, Bt, Js, their coefficients and
 // CPML memories -- in registers for the whole launch; neighbours meet in
 // shared memory, two barriers per step.  The launch reads one buffer and
@@ -102,7 +104,11 @@ __global__ void __launch_bounds__(kNT, 1) k_narrow(const __grid_constant__ Narro
         live = live && k >= 0 && k < P.N[2];
     }
     if (!live) k = 0;
-    const bool mine = live && kl >= A.steps && kl < A.steps + A.own && kw < P.N[2];
+    // a Mur wall goes with the plane next to it (with N[2] - 1 a multiple of `own`,
+    // or own = 1, it would be another CTA's, where that plane is spoiled by then)
+    const bool mur = P.bc[2] == TF_BC_MUR;
+    const int ko = (mur ? min(max(kw, 1), P.n[2] - 1) : kw) - (int)blockIdx.x * A.own;
+    const bool mine = live && ko >= 0 && ko < A.own && kw < P.N[2];
     // lanes that each component advances
     const Quad u = quad_of(P, x, j, k);
     const bool adv = live && (P.per[1] || j < P.n[1]) && (P.per[2] || k < P.n[2]);
@@ -122,7 +128,6 @@ __global__ void __launch_bounds__(kNT, 1) k_narrow(const __grid_constant__ Narro
     // First-order Mur: E of a wall plane comes from the plane next to it, whose
     // threads hold that plane's old and new E: they write the wall's as well,
     // its own threads only take it up
-    const bool mur = P.bc[2] == TF_BC_MUR;
     const bool wall = mur && live && (k == 0 || k == P.n[2]);
     const bool lo_wall = mur && live && k == 1 && kl > 0, hi_wall = mur && live && k == P.n[2] - 1 && kl + 1 < A.window;
     const bool by_wall = lo_wall || hi_wall;
@@ -394,7 +399,7 @@ __global__ void __launch_bounds__(kNT, 1) k_narrow(const __grid_constant__ Narro
 }
 
 cudaError_t launch_narrow(const NarrowArgs& A, const Probes& R, cudaStream_t st) {
-    const int blocks = (A.P.N[2] + A.own - 1) / A.own;
+    const int blocks = narrow_blocks(A.P, A.own);
     const int dft = A.steps_before > 0 ? (R.n * TF_MAX_FREQS + kNT / 32 - 1) / (kNT / 32) : 0;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(blocks + dft);
