@@ -529,14 +529,14 @@ tf_status tf64_set_materials(tf64_handle h, const double* eps_r, const double* m
     const long long nc = (long long)g.n[0] * g.n[1] * g.n[2];
     double* hc = (double*)malloc(sizeof(double) * 4 * (size_t)nc);
     if (!hc) return TF_ENOMEM;
-    g.uniform_mu = 1;
+    int uniform_mu = 1;   // (the handle's own follows with the coefficients: a refused call leaves both)
     for (long long m = 0; m < nc; ++m) {
         const double e = eps_r ? eps_r[m] : 1.0, u = mu_r ? mu_r[m] : 1.0;
         const double l = lambda_L ? lambda_L[m] : 0.0, s = sigma ? sigma[m] : 0.0;
         if (!(e > 0) || !(u > 0) || !(s >= 0) || l < 0) { free(hc); return TF_EINVAL; }
         hc[m] = e;
         hc[nc + m] = u;
-        if (u != 1.0) g.uniform_mu = 0;
+        if (u != 1.0) uniform_mu = 0;
         hc[2 * nc + m] = (l > 0 && isfinite(l)) ? 1.0 / (l * l * kMu0d * u) : 0.0;
         hc[3 * nc + m] = s;
     }
@@ -551,6 +551,7 @@ tf_status tf64_set_materials(tf64_handle h, const double* eps_r, const double* m
     k64_coeffs<<<blocks(g), kT, 0, h->st>>>(g);
     C64(cudaGetLastError());
     C64(cudaStreamSynchronize(h->st));
+    g.uniform_mu = uniform_mu;
     return TF_OK;
 }
 
