@@ -160,8 +160,11 @@ template <bool kEarly>
 __device__ __forceinline__ void pre_e(const PassArgs& A, const Quad& u, PreE& r) {
     const Params& P = A.P;
     r.rec = __ldg(A.tilemat + (long long)((u.j / kSY) * A.ntx + u.x / kSX) * P.N[2] + u.k);
-    r.ex = own4(P.E[0], u.o);
-    r.ey = own4(P.E[1], u.o);
+    // Ex and Ey of the low z wall are held, or a Mur update's, by the threads of
+    // the plane above during this very pass: none of this one's business
+    const Q4 z = {{0, 0}};
+    r.ex = u.inz ? own4(P.E[0], u.o) : z;
+    r.ey = u.inz ? own4(P.E[1], u.o) : z;
     r.ez = own4(P.E[2], u.o);
     if (u.sz) {
         r.p0 = own4(P.psiE[0][2], u.o);
