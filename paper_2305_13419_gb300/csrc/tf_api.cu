@@ -26,6 +26,7 @@ struct Layout {
     size_t off_fields, off_maps, off_psi, off_prof, off_zero, off_probe, off_series, off_scratch,
         off_tiles, off_order, off_order_s, off_order_t, off_stats, off_coef, off_samples, off_misc, bytes;
     int psa, psb, psc, pnbx, pnby, pnbz;   // items of the steps in place: 2^sa quads x 2^sb rows x 2^sc planes
+    int pwin;               // planes they take at a time (window_planes)
     long long max_s, max_t;   // capacity of the shell and two-step work lists
     long long scratch_floats;
     int nstat;              // partials of the statistics
@@ -66,9 +67,12 @@ tf_status validate(const tf_grid_desc* d) {
 // Shape of the items of the steps in place (a thread has a quad of x points):
 // the fewest threads off the grid; long rows before square ones (with rows of
 // 4 instead of 16 quads a step of the 512 x 256 x 128 CPW took 268 us instead
-// of 251); then few neighbours outside the item along y and z.
+// of 251); then few neighbours outside the item along y and z.  Items fill the
+// planes of a window, whose neighbours along z are in L2 all the same (us a step
+// with items of 4 planes / of one: 512 x 256 x 128 CPW 196 / 189, 900 x 400 x 200
+// CPW 943 / 904, 640 x 640 x 190 846 / 807).
 void pass_shape(Layout& L, int cx, int cy) {
-    const int nq = (cx + 3) / 4;
+    const int nq = (cx + 3) / 4, nz = L.pwin;
     L.psa = 0;
     L.psb = kPassBits;
     L.psc = 0;
@@ -76,10 +80,10 @@ void pass_shape(Layout& L, int cx, int cy) {
     for (int a = 0; a <= 4; ++a)
         for (int b = 0; a + b <= kPassBits; ++b) {
             const int c = kPassBits - a - b;
-            if (c > 0 && (1 << (c - 1)) >= L.kend) continue;
+            if (c > 0 && (1 << (c - 1)) >= nz) continue;
             if ((cy - 1) >> b > 65534 || (L.kend - 1) >> c > 65534) continue;   // a launch's y and z end there
-            const double full = (double)(((nq - 1) >> a) + 1) * (((cy - 1) >> b) + 1) * (((L.kend - 1) >> c) + 1);
-            const double halo = 1.0 + 1.2 / (1 << a) + 0.25 / (1 << b) + 0.25 / (1 << c);
+            const double full = (double)(((nq - 1) >> a) + 1) * (((cy - 1) >> b) + 1) * (((nz - 1) >> c) + 1);
+            const double halo = 1.0 + 1.2 / (1 << a) + 0.25 / (1 << b) + (nz < L.kend ? 0.0 : 0.25 / (1 << c));
             const double cost = full * halo;
             if (cost < best) {
                 best = cost;
@@ -136,6 +140,7 @@ Layout layout_of(const tf_grid_desc* d) {
     L.off_order_t = o; o += align_up(sizeof(long long) * (size_t)L.max_t);
     L.nstat = L.N[2] > kStatPartials ? L.N[2] : kStatPartials;
     L.off_stats = o;  o += align_up(sizeof(StatPartial) * (size_t)(L.nstat + 1));
+    L.pwin = window_planes(cx, cy, L.kend, d->bc[2].kind == TF_BC_PERIODIC);
     pass_shape(L, cx, cy);
     L.off_samples = o; o += align_up(2 * sizeof(float) * kPassSteps * TF_MAX_PROBES);   // two groups of steps
     L.off_misc = o;   o += kAlign;
@@ -741,6 +746,7 @@ PassArgs pass_args(const tf_ctx* h, const Sources& S) {
     A.cx = h->P.per[0] ? h->P.N[0] : h->P.n[0];
     A.cy = h->P.per[1] ? h->P.N[1] : h->P.n[1];
     A.kend = L.kend;
+    A.win = L.pwin;
     A.sms = h->sms;
     A.samples = (float*)(h->ws + L.off_samples);
     A.nprobe = h->R.n;

@@ -347,6 +347,22 @@ cudaError_t launch_step_advance(int* step, cudaStream_t st);
 constexpr int kPassSteps = 32;     // steps per group of launches (probe samples are kept for that many)
 constexpr long long kPassPoints = 80LL << 20;   // padded points of a grid up to which tf_step runs in place
 constexpr int kPassBits = 7, kPassThreads = 1 << kPassBits;   // threads of an item, a quad of x points each
+// Planes that a pass takes at a time, kend where it takes the grid whole (the
+// windows of tf_pass.cu, which has the figures).  Windows of fewer than four
+// planes lose to whole passes: a window moves down a plane per step, so one of p
+// planes finds p - 1 of them in L2.  us a step whole / in windows of 1 to 3 planes:
+// 1448 x 1448 x 38 1047 / 1327, 2000 x 1000 x 20 563 / 851, 1000 x 1000 x 80 992 /
+// 1176, 4000 x 4000 x 4 705 / 1065, 1000 x 1000 x 4 50 / 65, 800 x 800 x 100 784 /
+// 809; of 4: 700 x 700 x 80 488 / 446, 1024 x 512 x 100 643 / 584.
+constexpr double kWindowPoints = 1.9e6, kWindowMin = 2.8e6;
+constexpr int kWindowPlanes = 4;
+inline int window_planes(int cx, int cy, int kend, bool periodic_z) {
+    const double points = (double)cx * cy * kend;
+    if (periodic_z || points < kWindowMin) return kend;
+    const int n = (int)(points / kWindowPoints + 0.5), count = n < 2 ? 2 : n < kend ? n : kend;
+    const int planes = (kend + count - 1) / count;
+    return planes < kWindowPlanes ? kend : planes;
+}
 struct PassArgs {
     Params P;
     Sources S;                                  // amplitudes come from PassAmps
@@ -356,6 +372,7 @@ struct PassArgs {
     int sa, sb, sc;                             // an item: 2^sa quads x 2^sb rows x 2^sc planes
     int nbx, nby, nbz;                          // items along x, y, z
     int cx, cy, kend;                           // points advanced along x, y, z: [0, c)
+    int win;                                    // planes of a window (window_planes)
     int sms;                                    // multiprocessors of the device
     int nprobe;
     int pr_item[TF_MAX_PROBES], pr_k[TF_MAX_PROBES];   // the item along x, y and the plane that sample a probe

@@ -380,7 +380,7 @@ __device__ __forceinline__ void sample(const PassArgs& A, int t, int k0, int k1)
 // of its one round of loads on small grids (two launches, 7.5 us a step on the
 // 128 x 64 x 40 CPW) and by memory on large ones: over the whole 512 x 256 x 128
 // CPW it takes 234 us a step (6.2 TB/s of 72 bytes per point plus the CPML
-// memories), 199 in windows of planes (windows_of below: L2 to SM traffic and the
+// memories), 199 in windows of planes (below: L2 to SM traffic and the
 // launches' ends), on the 256 x 128 x 64 CPW, whose 90 MB nearly stay in L2, 31.  What is spilled goes to
 // L2 and back: with all three slab axes' memories and Js fetched up front the E
 // pass spilled 170 bytes a thread (252 and 43 us); now the first slab axis is
@@ -460,17 +460,14 @@ cudaError_t launch_pass_probes(const Probes& R, const float* samples, long long 
 //   160 x 160 x 128    53 / 1: 48, 1.4: 44, 1.8: 42;   128^3  30 / 1: 38, 1.4: 30
 // smaller windows leave the last wave of each launch emptier, larger ones leave
 // L2.  8 steps instead of 16 are 1 to 3 % slower, 4 steps 4 to 7 %.
-constexpr double kWindowPoints = 1.9e6, kWindowMin = 2.8e6;
+// Items of one plane: with items of 2 or 4 planes a window of 5 leaves a fifth to
+// two fifths of the threads idle (1024 x 400 x 180: 756 us a step against 900).
 constexpr int kWindowSteps = 16;
-struct Windows {
-    int planes, depth;
-};
-Windows windows_of(const PassArgs& A, int steps) {
-    const double points = (double)A.cx * A.cy * A.kend;
-    if (A.P.per[2] || points < kWindowMin) return {A.kend, 1};
-    const int most = A.kend < 1 << 20 ? A.kend : 1 << 20, n = (int)(points / kWindowPoints + 0.5);
-    const int count = n < 2 ? 2 : n < most ? n : most, groups = (steps + kWindowSteps - 1) / kWindowSteps;
-    return {(A.kend + count - 1) / count, (steps + groups - 1) / groups};
+// steps of a window, of `steps` in all: groups of one size
+int window_steps(const PassArgs& A, int steps) {
+    if (A.win == A.kend) return 1;
+    const int groups = (steps + kWindowSteps - 1) / kWindowSteps;
+    return (steps + groups - 1) / groups;
 }
 
 // `steps` steps from `level`, two launches per step and window of planes, with
@@ -488,14 +485,14 @@ cudaError_t launch_passes(const PassArgs& A, const Probes& R, const PassAmps* am
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     const bool early = A.nbx * A.nby * A.nbz <= kEarlyMin * A.sms;
-    const Windows win = windows_of(A, steps);
+    const int depth = window_steps(A, steps);
     cfg.numAttrs = 0;   // the first launch waits for whatever the stream holds
     cudaError_t e = cudaSuccess;
-    for (int t0 = 0; t0 < steps; t0 += win.depth) {
-        const int m = steps - t0 < win.depth ? steps - t0 : win.depth;
-        for (int z = 0; z < A.kend + m - 1; z += win.planes)
+    for (int t0 = 0; t0 < steps; t0 += depth) {
+        const int m = steps - t0 < depth ? steps - t0 : depth;
+        for (int z = 0; z < A.kend + m - 1; z += A.win)
             for (int u = 0; u < m && e == cudaSuccess; ++u) {
-                const int k0 = z > u ? z - u : 0, k1 = z + win.planes - u < A.kend ? z + win.planes - u : A.kend;
+                const int k0 = z > u ? z - u : 0, k1 = z + A.win - u < A.kend ? z + A.win - u : A.kend;
                 if (k0 >= k1) continue;
                 const PassAmps& W = amp[t0 + u];
                 cfg.gridDim.z = ((k1 - k0 - 1) >> A.sc) + 1;
