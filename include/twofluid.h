@@ -158,8 +158,9 @@ tf_status tf_add_probe(tf_handle h, int comp, const int p[3], const double* freq
  * update with CPML memory, the Js update, the theta-scheme E update with
  * sources, the Mur walls, the probe DFTs and the non-finite watchdog.  Grids
  * of up to some 80 million points run in place, a B pass and an E pass per
- * step; larger ones one fused launch per step or two-step passes
- * (tf_set_two_step).  The results are the same bits.  Asynchronous; launch errors are
+ * step, but for large ones that two-step passes (tf_set_two_step) step faster;
+ * larger ones take those or one fused launch per step.  The results are the
+ * same bits.  Asynchronous; launch errors are
  * returned (the handle is then unusable), device-side errors latch for
  * tf_sync(). */
 tf_status tf_step(tf_handle h, int64_t nsteps);
@@ -193,7 +194,7 @@ tf_status tf_step_timed(tf_handle h, int64_t nsteps, double* kernel_ms, int64_t*
  * same bits as single steps.  It is used when the box is not empty, mu is
  * uniform (tf_set_materials) and it is enabled; an odd step count ends with a
  * single step.  By default tf_step takes it on grids too large to run in
- * place.
+ * place, and on large ones that are slower in place.
  *   tf_set_two_step  planes = 0 disables it for this handle; 4 .. 24 asks for
  *                    it, with work items of that many planes (24 by default),
  *                    also on grids that would run in place;

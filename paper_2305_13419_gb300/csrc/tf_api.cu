@@ -201,7 +201,8 @@ struct tf_ctx {
     char* ws;
     float* scratch;
     unsigned* status;
-    unsigned* mm;      // 4 words: max 1/(eps mu), max kt/(4 eps), non-uniform mu, spare
+    unsigned* mm;      // 4 words: max 1/(eps mu), max kt/(4 eps), non-uniform mu, tile-planes of varying material
+    double varying;    // the share of such tile-planes
     double* fit_out;   // 4 doubles
     int nsrc;
     SrcHost src[TF_MAX_SOURCES];
@@ -497,7 +498,7 @@ tf_status tf_create(const tf_grid_desc* desc, void* dev_workspace, size_t bytes,
     if (e == cudaSuccess)
         e = launch_convert_materials(P, nullptr, nullptr, nullptr, nullptr, dt, maps[0], maps[1], maps[2],
                                      maps[3], h->mm, h->stream);
-    if (e == cudaSuccess) e = launch_tile_materials(P, (float4*)O.tilemat, L.ntx, L.nty, h->stream);
+    if (e == cudaSuccess) e = launch_tile_materials(P, (float4*)O.tilemat, L.ntx, L.nty, h->mm + 3, h->stream);
     if (e == cudaSuccess) e = launch_edge_coeffs(P, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) { delete h; return TF_ECUDA; }
@@ -553,7 +554,7 @@ tf_status tf_set_materials(tf_handle h, const float* eps_r, const float* mu_r, c
     TF_CUDA(cudaMemsetAsync(h->status, 0, sizeof(unsigned), h->stream));
     TF_CUDA(launch_convert_materials(P, dev[0], dev[1], dev[2], dev[3], h->dt, (float*)P.eps, (float*)P.sig,
                                      (float*)P.kap, (float*)P.mu, h->mm, h->stream));
-    TF_CUDA(launch_tile_materials(P, (float4*)h->O.tilemat, h->L.ntx, h->L.nty, h->stream));
+    TF_CUDA(launch_tile_materials(P, (float4*)h->O.tilemat, h->L.ntx, h->L.nty, h->mm + 3, h->stream));
     h->order_dirty = 1;
     TF_CUDA(launch_edge_coeffs(P, h->stream));
     TF_CUDA(launch_mask_js(P, h->stream));
@@ -563,6 +564,7 @@ tf_status tf_set_materials(tf_handle h, const float* eps_r, const float* mu_r, c
     TF_CUDA(cudaStreamSynchronize(h->stream));
     TF_CUDA(cudaMemsetAsync(h->status, 0, sizeof(unsigned), h->stream));
     P.uniform_mu = hm[2] ? 0 : 1;
+    h->varying = (double)hm[3] / ((double)h->L.ntx * h->L.nty * h->L.N[2]);
     if (!P.uniform_mu) {
         TF_CUDA(launch_face_imu(P, h->fE[2], h->stream));
         h->imu_kept = 1;
@@ -867,16 +869,45 @@ cudaError_t run_narrow(tf_ctx* h, const Sources& S, int64_t nsteps) {
     return e;
 }
 
-// Does tf_step run in place (tf_pass.cu)?  Not when two-step passes were
-// asked for, nor under a wait limit of the handle's own (the passes wait for
-// nothing).  us per step in place / single staged steps / two-step passes on
-// CPW grids: 0.3 M cells 7.5 / 21 / 68, 2.1 M 31 / 72 / 126, 4 M 56 / 104 / 149,
-// 8 M 102 / 165 / 182, 17 M 199 / 266 / 273, 32 M 368 / - / 421, 72 M 945 / - /
-// 970, 134 M 1620 / 1695 / 1512: planes of half a million points leave a window
-// of planes (tf_pass.cu) too little of L2.
+// Two-step passes of staged planes against steps in place, where both may run: on
+// large grids whose passes are whole (a periodic z axis, or planes too large for
+// windows) they are faster, less by what the CPML slabs, the walls of a thin box
+// and per-point coefficients add to them.  With N million cells, s the slabs' share
+// of the cells along x and y / z, v that of the tile-planes with per-point
+// coefficients, whole passes take some 11 N us a step and two-step passes
+// 8.4 N + 50 plus the rest: a gain of about N (2.6 - 10 s_xy - 4 s_z - 6 v) - 50,
+// where nothing wraps along x (tiles next to a seam there are slow).  In place /
+// two-step, whole passes: 400^3 periodic along z with CPML 795 / 729, 300^3 355 /
+// 362, 1024 x 512 x 128 774 / 663, 512 x 256 x 128 209 / 217, with walls 512 x 512 x
+// 200 578 / 496, 256 x 256 x 300 217 / 215, 512 x 512 x 256 periodic throughout 729 /
+// 1056; 1448 x 1448 x 38 CPML 1047 / 1002, 2000 x 1500 x 24 978 / 1011, 31 M cells of
+// random material 650 / 831.  Windows of planes beyond some 0.45 M points lose a
+// little as well, with CPML: 1024 x 512 x 150 831 / 810, 720 x 720 x 110 610 / 591,
+// but 1024 x 512 x 100 568 / 577, with walls 1024 x 512 x 150 685 / 718 (smaller
+// planes: 640 x 640 x 190 809 / 818, 900 x 400 x 200 CPW 906 / 969).
+bool two_step_pays(const tf_ctx* h) {
+    const Params& P = h->P;
+    if (!h->two_step_on || !h->box_ok || !P.uniform_mu || P.per[0]) return false;
+    const double cells = (double)h->L.ncell, plane = (double)P.n[0] * P.n[1];
+    const double box = (double)(h->tx1 - h->tx0) * kSX * (h->ty1 - h->ty0) * kSY * (h->tz1 - h->tz0);
+    if (box < 0.5 * cells) return false;
+    const double sxy = 2.0 * P.L[0] / P.n[0] + 2.0 * P.L[1] / P.n[1], sz = 2.0 * P.L[2] / P.n[2];
+    const double gain = 1e-6 * cells * (2.6 - 10.0 * sxy - 4.0 * sz - 6.0 * h->varying);
+    return h->L.pwin == h->L.kend ? gain > 50.0 : plane > 4.5e5 && sxy > 0.0 && gain > 100.0;
+}
+
+// May steps in place take the grid (tf_pass.cu)?  Not under a wait limit of the
+// handle's own (the passes wait for nothing), nor above kPassPoints: us a step in
+// place / in two-step passes on a CPW grid of 134 M cells 1620 / 1512.
+bool may_pass(const tf_ctx* h) { return h->P.wait_polls == kSpinLimit && h->L.total <= kPassPoints; }
+
+// Does tf_step run in place?  Not when two-step passes were asked for.  us per step
+// in place / single staged steps / two-step passes on CPW grids: 0.3 M cells 7.5 /
+// 21 / 68, 2.1 M 31 / 72 / 126, 4 M 56 / 104 / 149, 8 M 101 / 165 / 182, 17 M 189 /
+// 266 / 272, 32 M 364 / - / 448, 72 M 906 / - / 969.
 bool in_place(const tf_ctx* h) {
     const bool asked = h->two_step_on == 2 && h->box_ok && h->P.uniform_mu;
-    return !asked && h->P.wait_polls == kSpinLimit && h->L.total <= kPassPoints;
+    return !asked && may_pass(h) && !two_step_pays(h);
 }
 
 bool two_step(const tf_ctx* h) { return h->two_step_on && h->box_ok && h->P.uniform_mu && h->nitems_t > 0; }
@@ -1200,10 +1231,11 @@ struct BatchStreams {
     }
 };
 
-// a batch runs grid by grid where every grid may step in place
+// a batch runs grid by grid where every grid may step in place (against one launch
+// of single staged steps, which whole passes beat as well)
 bool batch_in_place(const tf_handle* hs, int n) {
     for (int i = 0; i < n; ++i)
-        if (hs[i]->P.wait_polls != kSpinLimit || hs[i]->L.total > kPassPoints) return false;
+        if (!may_pass(hs[i])) return false;
     return true;
 }
 
@@ -1801,7 +1833,7 @@ tf_status tf_adjoint_run(tf_handle h, int64_t nsteps, int probe, int freq_index,
         const int64_t len = seg_len(s);
         float* const d0[3] = {hist(s, 0, 0), hist(s, 0, 1), hist(s, 0, 2)};
         TF_CUDA(launch_copy3(d0, h->P.E, h->L.total, h->stream));
-        if (in_place(h)) {   // the E passes write the history as well
+        if (may_pass(h)) {   // the E passes write the history as well
             if (!h->primed) {
                 TF_CUDA(launch_prime(h->P, h->stream));
                 h->primed = 1;

@@ -449,7 +449,7 @@ cudaError_t launch_step(const void* tmaps, const Params& P, const StepOut& O, co
                         long long n, int blocks, cudaStream_t st);
 cudaError_t launch_edge_coeffs(const Params& P, cudaStream_t st);
 size_t step_smem_bytes();
-cudaError_t launch_tile_materials(const Params& P, float4* tilemat, int ntx, int nty, cudaStream_t st);
+cudaError_t launch_tile_materials(const Params& P, float4* tilemat, int ntx, int nty, unsigned* varying, cudaStream_t st);
 // discrete adjoint (tf_adjoint.cu): the adjoint state, in the scaled units of
 // the step, and per-edge gradient sums (FP64)
 struct AdjState {

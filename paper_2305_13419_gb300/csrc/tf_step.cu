@@ -1056,10 +1056,11 @@ __global__ void __launch_bounds__(kThreads, 2)
 
 // per (tile, plane): are all cells an owned edge or face of the tile-plane
 // touches alike?  Then store {ca, cb, cj, 1/mu}; else ca = NaN, and 1 or 0 for
-// "no conducting cell: ca = 1 on every edge" and "a superconducting cell".
+// "no conducting cell: ca = 1 on every edge" and "a superconducting cell",
+// and count it in `varying`.
 // (A plane per CTA: tiles that walked their planes one by one took three
 // barriers and a round of loads for each.)
-__global__ void k_tile_materials(Params P, float4* rec, int ntx, int nty) {
+__global__ void k_tile_materials(Params P, float4* rec, int ntx, int nty, unsigned* varying) {
     const int bx = blockIdx.x, by = blockIdx.y;
     const int tid = threadIdx.y * blockDim.x + threadIdx.x, nth = blockDim.x * blockDim.y;
     auto cellc = [&](int a, int v) {
@@ -1094,6 +1095,7 @@ __global__ void k_tile_materials(Params P, float4* rec, int ntx, int nty) {
                 r = make_float4((e0 - (1.f - P.theta) * s0) / den, 1.f / den, k0, 1.f / u0);
             } else {
                 r = make_float4(__int_as_float(0x7fc00000), cond ? 0.f : 1.f, super ? 1.f : 0.f, 0.f);
+                atomicAdd(varying, 1u);
             }
             rec[(long long)(by * ntx + bx) * P.N[2] + k] = r;
         }
@@ -1268,8 +1270,8 @@ cudaError_t launch_item_order(const Params& P, const StepOut& O, const Sources& 
     return cudaGetLastError();
 }
 
-cudaError_t launch_tile_materials(const Params& P, float4* rec, int ntx, int nty, cudaStream_t st) {
-    k_tile_materials<<<dim3(ntx, nty, P.N[2] < 65535 ? P.N[2] : 65535), dim3(32, 8), 0, st>>>(P, rec, ntx, nty);
+cudaError_t launch_tile_materials(const Params& P, float4* rec, int ntx, int nty, unsigned* varying, cudaStream_t st) {
+    k_tile_materials<<<dim3(ntx, nty, P.N[2] < 65535 ? P.N[2] : 65535), dim3(32, 8), 0, st>>>(P, rec, ntx, nty, varying);
     return cudaGetLastError();
 }
 

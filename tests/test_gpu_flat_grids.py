@@ -24,3 +24,38 @@ def test_flat_grids_give_the_bits_of_staged_steps(case):
         g.step(n)
     g.sync()
     _same(g, ref, w, 41)
+
+
+@pytest.mark.parametrize("n,bc,varying,two", [((512, 512, 128), (C, C, P), False, True), ((512, 512, 128), (C, C, P), True, False),
+                                              ((256, 512, 128), (C, C, P), False, False), ((512, 512, 128), (P, C, P), False, False),
+                                              ((800, 800, 80), (W_, W_, W_), False, True), ((512, 512, 128), (C, C, C), False, False),
+                                              ((1000, 1000, 30), (C, C, C), False, False)])
+def test_where_two_step_passes_pay(n, bc, varying, two):
+    """tf_step's choice between steps in place and two-step passes where
+    neither was asked for, and the same bits either way."""
+    from paper_2305_13419_gb300 import twofluid as tf
+    from paper_2305_13419_gb300 import workloads as W
+    d = (10e-9, 12e-9, 8e-9)
+    cpml = tuple(W.default_cpml(6, d[a], 1e12) if bc[a] == C else None for a in range(3))
+    grids = []
+    for default in (True, False):
+        gen = torch.Generator(device="cuda").manual_seed(5)
+        g = tf.Grid(n, d, 1.0, bc, cpml, courant=0.9)
+        cells = (n[2], n[1], n[0])
+        eps = torch.full(cells, 2.5, device="cuda")
+        if varying:
+            eps += torch.rand(cells, generator=gen, device="cuda")
+        g.set_materials(eps, torch.ones_like(eps), torch.zeros_like(eps), torch.zeros_like(eps))
+        if not default:
+            g.set_two_step(False)
+        for c in range(6):
+            g.set_field(c, (torch.rand(g.shape, generator=gen, device="cuda") - 0.5) * W.FIELD_SCALE[c])
+        g.step(5)
+        g.sync()
+        grids.append(g)
+    assert [g.two_step_box()[1] for g in grids] == [two, False]
+    a, b = (torch.empty(g.shape, device="cuda") for g in grids)
+    for c in range(6):
+        grids[0].field(c, out=a)
+        grids[1].field(c, out=b)
+        assert torch.equal(a, b), c
