@@ -154,26 +154,34 @@ __global__ void k_prime(Params P) {
     }
 }
 
-// v * scale to FP32's rounding, the scale as an unevaluated sum of two FP32
-// numbers: the product's error enters before the one rounding that counts
-// (against FP64 arithmetic it rounds the other way on one value in some 2^22;
-// three FP32 operations where the FP64 pipe takes 48 cycles per warp)
-__device__ __forceinline__ float scaled(float v, float sh, float sl) {
-    const float p = __fmul_rn(v, sh);
-    return isfinite(p) ? __fadd_rn(p, __fmaf_rn(v, sl, __fmaf_rn(v, sh, -p))) : p;
+// (float)(v * scale) of FP64 arithmetic, whose pipe takes 48 cycles per warp, with
+// FP32's: the scale as an unevaluated sum sh + sl, the product as p + t.  t is off
+// by less than 2^-20 of itself, but where it is too small to matter; if p + t
+// rounds to the same number either side of that, so does the FP64 product.  The
+// others (some four in ten million), and what is no normal number or has too few
+// bits below it for t, take the FP64 pipe.
+struct Scale {
+    float sh, sl;
+    double s;
+};
+__device__ __forceinline__ float scaled(float v, const Scale& S) {
+    const float p = __fmul_rn(v, S.sh), t = __fmaf_rn(v, S.sl, __fmaf_rn(v, S.sh, -p));
+    const float lo_ = __fmaf_rn(t, 1.f - 0x1p-20f, p), hi_ = __fmaf_rn(t, 1.f + 0x1p-20f, p);
+    const bool sure = lo_ == hi_ && fabsf(p) > 0x1p-100f && fabsf(p) < 0x1p127f;
+    return sure ? hi_ : v == 0.f ? p : (float)((double)v * S.s);
 }
 
 // integer-level value of component c of E (kKind 0), B (1) or Js (2) at a point
 template <int kKind>
 __device__ __forceinline__ float read_point(const Params& P, int c, int primed, const float4* tilemat, int ntx,
-                                            const int p[3], float sh, float sl) {
+                                            const int p[3], const Scale& S) {
     const int q = (int)lin(P, p[0], p[1], p[2]);
     if constexpr (kKind == 0) {
         return P.E[c][q];
     } else if constexpr (kKind == 1) {
         float b = P.B[c][q];
         if (primed && upd_B(P, c, p)) b -= 0.5f * curl_E_peek(P, c, p, q);
-        return scaled(b, sh, sl);
+        return scaled(b, S);
     } else {
         // Js lives on superconducting edges only: none on a tile-plane
         // without a superconducting cell, nor off the tiles (walls)
@@ -182,14 +190,14 @@ __device__ __forceinline__ float read_point(const Params& P, int c, int primed, 
         if (!(rec.z > 0.f)) return 0.f;
         const float kt = __ldg(P.cj[c] + q);   // zero on the other edges and on edges no step advances
         if (!(kt > 0.f)) return 0.f;
-        return scaled(P.J[c][q] + (primed ? 0.5f * kt * P.E[c][q] : 0.f), sh, sl);
+        return scaled(P.J[c][q] + (primed ? 0.5f * kt * P.E[c][q] : 0.f), S);
     }
 }
 
 // four points of a row of B_c (32 apart, from i0): every load that all points
 // need before the first use, at positions kept inside the row
 template <int kC>
-__device__ __forceinline__ void read_b_row(const Params& P, int primed, int i0, int j, int k, float sh, float sl, float v[4]) {
+__device__ __forceinline__ void read_b_row(const Params& P, int primed, int i0, int j, int k, const Scale& S, float v[4]) {
     constexpr int a1 = kC == 0 ? 1 : 0, a2 = kC == 2 ? 1 : 2;
     const float *e1 = P.E[3 - kC - a1], *e2 = P.E[3 - kC - a2];
     const int row = (int)lin(P, 0, j, k);
@@ -214,7 +222,7 @@ __device__ __forceinline__ void read_b_row(const Params& P, int primed, int i0, 
                 t2 += P.pbB[a2][p[a2]] * P.psiB[kC][a2][q] + P.pcB[a2][p[a2]] * d2[u];
             v[u] -= 0.5f * (curl_sign(kC, a1) * t1 + curl_sign(kC, a2) * t2);
         }
-        v[u] = scaled(v[u], sh, sl);
+        v[u] = scaled(v[u], S);
     }
 }
 
@@ -228,19 +236,19 @@ __device__ __forceinline__ void read_b_row(const Params& P, int primed, int i0, 
 // kRows = false: rows shorter than a warp, points in sequence.
 template <int kKind, int kC, bool kRows>
 __global__ void __launch_bounds__(256) k_read_field(Params P, int primed, const float4* tilemat, int ntx,
-                                                    float* dense, float sh, float sl) {
+                                                    float* dense, Scale S) {
     if constexpr (kRows) {
         const int j = blockIdx.y * 8 + threadIdx.y, k = blockIdx.z, i0 = blockIdx.x * 128 + threadIdx.x;
         if (j >= P.N[1]) return;
         float* const out = dense + ((long long)k * P.N[1] + j) * P.N[0];
         float v[4];
         if constexpr (kKind == 1) {
-            read_b_row<kC>(P, primed, i0, j, k, sh, sl, v);
+            read_b_row<kC>(P, primed, i0, j, k, S, v);
         } else {
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 const int p[3] = {i0 + 32 * u, j, k};
-                if (p[0] < P.N[0]) v[u] = read_point<kKind>(P, kC, primed, tilemat, ntx, p, sh, sl);
+                if (p[0] < P.N[0]) v[u] = read_point<kKind>(P, kC, primed, tilemat, ntx, p, S);
             }
         }
 #pragma unroll
@@ -249,7 +257,7 @@ __global__ void __launch_bounds__(256) k_read_field(Params P, int primed, const 
     } else {
         const unsigned t = blockIdx.x * 256u + threadIdx.x, row = t / (unsigned)P.N[0];
         const int p[3] = {(int)(t - row * (unsigned)P.N[0]), (int)(row % (unsigned)P.N[1]), (int)(row / (unsigned)P.N[1])};
-        if (p[2] < P.N[2]) dense[t] = read_point<kKind>(P, kC, primed, tilemat, ntx, p, sh, sl);
+        if (p[2] < P.N[2]) dense[t] = read_point<kKind>(P, kC, primed, tilemat, ntx, p, S);
     }
 }
 
@@ -314,36 +322,37 @@ cudaError_t launch_prime(const Params& P, cudaStream_t st) {
 }
 
 template <int kKind, int kC>
-static void read_kernel(const Params& P, int primed, const float4* tilemat, int ntx, float* dense, float sh, float sl,
+static void read_kernel(const Params& P, int primed, const float4* tilemat, int ntx, float* dense, const Scale& S,
                         cudaStream_t st) {
     if (P.N[0] >= 32 && P.N[1] <= 8 * 65535 && P.N[2] <= 65535) {   // (blockIdx.y and z end there)
         k_read_field<kKind, kC, true><<<dim3((P.N[0] + 127) / 128, (P.N[1] + 7) / 8, P.N[2]), dim3(32, 8), 0, st>>>(
-            P, primed, tilemat, ntx, dense, sh, sl);
+            P, primed, tilemat, ntx, dense, S);
     } else {
         const long long tot = (long long)P.N[0] * P.N[1] * P.N[2];
-        k_read_field<kKind, kC, false><<<blocks_for(tot, 256), 256, 0, st>>>(P, primed, tilemat, ntx, dense, sh, sl);
+        k_read_field<kKind, kC, false><<<blocks_for(tot, 256), 256, 0, st>>>(P, primed, tilemat, ntx, dense, S);
     }
 }
 template <int kKind>
-static void read_kernel_of(const Params& P, int c, int primed, const float4* tilemat, int ntx, float* dense, float sh,
-                           float sl, cudaStream_t st) {
+static void read_kernel_of(const Params& P, int c, int primed, const float4* tilemat, int ntx, float* dense,
+                           const Scale& S, cudaStream_t st) {
     if (c == 0)
-        read_kernel<kKind, 0>(P, primed, tilemat, ntx, dense, sh, sl, st);
+        read_kernel<kKind, 0>(P, primed, tilemat, ntx, dense, S, st);
     else if (c == 1)
-        read_kernel<kKind, 1>(P, primed, tilemat, ntx, dense, sh, sl, st);
+        read_kernel<kKind, 1>(P, primed, tilemat, ntx, dense, S, st);
     else
-        read_kernel<kKind, 2>(P, primed, tilemat, ntx, dense, sh, sl, st);
+        read_kernel<kKind, 2>(P, primed, tilemat, ntx, dense, S, st);
 }
 
 cudaError_t launch_read_field(const Params& P, int comp, int primed, const float4* tilemat, int ntx, float* dense,
                               double scale, cudaStream_t st) {
-    const float sh = (float)scale, sl = (float)(scale - (double)sh);
+    const float sh = (float)scale;
+    const Scale S = {sh, (float)(scale - (double)sh), scale};
     if (comp < 3)
-        read_kernel_of<0>(P, comp, primed, tilemat, ntx, dense, sh, sl, st);
+        read_kernel_of<0>(P, comp, primed, tilemat, ntx, dense, S, st);
     else if (comp < 6)
-        read_kernel_of<1>(P, comp - 3, primed, tilemat, ntx, dense, sh, sl, st);
+        read_kernel_of<1>(P, comp - 3, primed, tilemat, ntx, dense, S, st);
     else
-        read_kernel_of<2>(P, comp - 6, primed, tilemat, ntx, dense, sh, sl, st);
+        read_kernel_of<2>(P, comp - 6, primed, tilemat, ntx, dense, S, st);
     return cudaGetLastError();
 }
 
