@@ -26,8 +26,16 @@ inline dim3 grid_of(const Params& P) {
     return dim3((P.N[0] + BX - 1) / BX, (P.N[1] + BY - 1) / BY, (P.N[2] + BZ - 1) / BZ);
 }
 
-// component cb of curl E at the B_cb position of p (scaled units, r_a folded
-// in), with the CPML memory advanced to the current E without storing it
+// the term of axis a in component cb of curl E at point p, from its difference dE
+// (scaled units, r_a folded in), with the CPML memory advanced to the current E
+// without storing it.  Every rounding is spelled out, so that a value does not
+// depend on the kernel that reads it.
+__device__ __forceinline__ float curl_term(const Params& P, int cb, int a, int pa, long long q, float dE) {
+    const float t = __fmul_rn(P.r[a], dE);
+    if (!P.psiB[cb][a] || !in_slab(P, a, pa)) return t;
+    return __fadd_rn(t, __fmaf_rn(P.pbB[a][pa], P.psiB[cb][a][q], __fmul_rn(P.pcB[a][pa], dE)));
+}
+// component cb of curl E at the B_cb position of p
 __device__ __forceinline__ float curl_E_peek(const Params& P, int cb, const int p[3], long long q) {
     float acc = 0.f;
 #pragma unroll
@@ -37,10 +45,7 @@ __device__ __forceinline__ float curl_E_peek(const Params& P, int cb, const int 
         int pn[3] = {p[0], p[1], p[2]};
         pn[a] = nxt(P, a, p[a]);
         const float dE = P.E[e][lin(P, pn[0], pn[1], pn[2])] - P.E[e][q];
-        float t = P.r[a] * dE;
-        if (P.psiB[cb][a] && in_slab(P, a, p[a]))
-            t += P.pbB[a][p[a]] * P.psiB[cb][a][q] + P.pcB[a][p[a]] * dE;
-        acc += curl_sign(cb, a) * t;
+        acc = __fadd_rn(acc, curl_sign(cb, a) * curl_term(P, cb, a, p[a], q, dE));
     }
     return acc;
 }
@@ -180,7 +185,7 @@ __device__ __forceinline__ float read_point(const Params& P, int c, int primed, 
         return P.E[c][q];
     } else if constexpr (kKind == 1) {
         float b = P.B[c][q];
-        if (primed && upd_B(P, c, p)) b -= 0.5f * curl_E_peek(P, c, p, q);
+        if (primed && upd_B(P, c, p)) b = __fmaf_rn(-0.5f, curl_E_peek(P, c, p, q), b);
         return scaled(b, S);
     } else {
         // Js lives on superconducting edges only: none on a tile-plane
@@ -215,12 +220,9 @@ __device__ __forceinline__ void read_b_row(const Params& P, int primed, int i0, 
     for (int u = 0; u < 4; ++u) {
         const int p[3] = {min(i0 + 32 * u, P.N[0] - 1), j, k}, q = row + p[0];
         if (primed && upd_B(P, kC, p)) {   // curl_E_peek of the loaded differences
-            float t1 = P.r[a1] * d1[u], t2 = P.r[a2] * d2[u];
-            if (P.psiB[kC][a1] && in_slab(P, a1, p[a1]))
-                t1 += P.pbB[a1][p[a1]] * P.psiB[kC][a1][q] + P.pcB[a1][p[a1]] * d1[u];
-            if (P.psiB[kC][a2] && in_slab(P, a2, p[a2]))
-                t2 += P.pbB[a2][p[a2]] * P.psiB[kC][a2][q] + P.pcB[a2][p[a2]] * d2[u];
-            v[u] -= 0.5f * (curl_sign(kC, a1) * t1 + curl_sign(kC, a2) * t2);
+            const float t1 = curl_sign(kC, a1) * curl_term(P, kC, a1, p[a1], q, d1[u]);
+            const float t2 = curl_sign(kC, a2) * curl_term(P, kC, a2, p[a2], q, d2[u]);
+            v[u] = __fmaf_rn(-0.5f, __fadd_rn(__fadd_rn(0.f, t1), t2), v[u]);
         }
         v[u] = scaled(v[u], S);
     }

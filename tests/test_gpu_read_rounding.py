@@ -37,3 +37,38 @@ def test_conversion_to_si_is_rounded_once(dt, js, nx):
             held = (v.astype(np.float64) * to).astype(np.float32)
             want = (held.astype(np.float64) * (1.0 / C0 if comp < 6 else EPS0 / dt)).astype(np.float32)
         assert np.array_equal(g.field(comp), want, equal_nan=True), comp
+
+
+@pytest.mark.parametrize("bc", [("periodic", "periodic", "periodic"), ("pec", "periodic", "mur"), ("periodic", "pec", "pec")],
+                         ids="-".join)
+@pytest.mark.parametrize("nx", [7, 33, 140])
+def test_integer_level_b_rounds_every_product_and_sum(nx, bc):
+    """B^n = B^{n-1/2} - curl E / 2 of the stored arrays, formed in FP32 one
+    operation at a time, whichever kernel reads the row."""
+    from paper_2305_13419_gb300 import twofluid as tf
+    from paper_2305_13419_gb300 import workloads as W
+    w = W.random_box(n=(nx, 9, 11), bc=bc, seed=nx)
+    st = W.random_state(4, w.storage_dims())
+    g = tf.Grid.from_workload(w)
+    for c in range(9):
+        g.set_field(c, st[c].astype(np.float32))
+    g.step(2)
+    blob = g.save_checkpoint()
+    pitch = int(blob[20:24].view(np.int32)[0])   # after the magic and the three sizes
+    raw = blob[256:].view(np.float32)[:6 * pitch * g.N[1] * g.N[2]].reshape(6, g.N[2], g.N[1], pitch)[..., :g.N[0]]
+    E, B = raw[:3], raw[3:]
+    r = [np.float32(C0 * g.dt / w.d[a]) for a in range(3)]
+    for c in range(3):
+        acc = np.zeros(g.shape, np.float32)
+        held = np.zeros(g.shape, bool)
+        for a in range(3):
+            if bc[a] != "periodic":   # off the axis: the half positions; along it: off both walls
+                at = np.arange(g.N[a]).reshape([-1 if i == 2 - a else 1 for i in range(3)])
+                held |= (at == w.n[a]) | ((at == 0) if a == c else False)
+            if a == c:
+                continue
+            t = r[a] * (np.roll(E[3 - c - a], -1, 2 - a) - E[3 - c - a])
+            acc = acc + (t if (a - c) % 3 == 1 else -t)
+        b = np.where(held, B[c], B[c] - np.float32(0.5) * acc)
+        want = (b.astype(np.float64) * (1.0 / C0)).astype(np.float32)
+        assert np.array_equal(g.field(3 + c), want), c
