@@ -380,6 +380,48 @@ def roofline_of(w, g, kt, planes=24, item_planes=8):
                 "kernel_ms": {k: v[0] for k, v in kt.items()}}
 
 
+def steps_in_place(g):
+    """Does tf_step run this grid in place (no two-step passes, no more padded
+    points than it takes there)?"""
+    pitch = (g.N[0] + 1 + 31) // 32 * 32
+    return not g.two_step_box()[1] and pitch * g.N[1] * g.N[2] <= 80 << 20
+
+
+def roofline_in_place(w, g, ms_per_step):
+    """Roofline of steps in place: a step's one-pass bytes over its time (the
+    launches of a step overlap, so they are not timed apart)."""
+    peak, peak_kind = hbm_peak()
+    ab = algorithmic_bytes(w, g.N)
+    # many steps per launch on planes of up to 32 quads of points
+    narrow = (g.N[0] + 3) // 4 * g.N[1] <= 32 and w.bc[0] != "cpml" and w.bc[1] != "cpml" and np.all(w.mu_r == 1)
+    gbs = ab["step"] / (ms_per_step * 1e-3) / 1e9
+    dense = ab["dense_equivalent"] / (ms_per_step * 1e-3) / 1e9
+    return ab, {"bound": "hbm", "kernel": "k_narrow" if narrow else "k_pass", "achieved": gbs, "peak": peak,
+                "unit": "GB/s", "frac": gbs / peak, "traffic": None, "algorithmic_bytes": ab["step"],
+                "peak_source": f"{peak_kind} (MEASURED_PEAKS.json hbm_gbs)" if peak_kind == "measured" else "fallback",
+                "dense_equivalent_GBps": dense, "effective_frac_dense_equivalent": dense / peak}
+
+
+def timed_steps(g, steps):
+    """`steps` steps of what tf_step runs: ms, and the kernels' own times where
+    it runs staged kernels (None in place)."""
+    if steps_in_place(g):
+        return g.time_steps(steps), None
+    kt, ms = g.step_timed(steps, with_total=True)
+    return ms, kt
+
+
+def roofline_of_run(w, g, steps, ms, kt, tuning, item_planes=8):
+    """(algorithmic bytes, roofline, launches of the stepping kernels: in place
+    at least two per step) of a timed_steps run."""
+    if kt is None:
+        ab, roof = roofline_in_place(w, g, ms / steps)
+        return ab, roof, -(-steps // 32) if roof["kernel"] == "k_narrow" else 2 * steps
+    ab, roof = roofline_of(w, g, kt, planes=tuning["best"] if tuning and tuning["best"] else 24,
+                           item_planes=tuning["item_planes"] if tuning else item_planes)
+    return ab, roof, sum(v[1] for v in kt.values())
+
+
 # ------------------------------------------------------------------ our arm
 def run_ours(args, ws, rank, local):
     import torch
@@ -404,24 +446,23 @@ def run_ours(args, ws, rank, local):
     N = g.N
 
     # device-timed throughput: inputs resident in HBM, K steps between
-    # barriers; CUDA events on the grid's stream around every launch, so the
-    # whole run and the kernel's own durations come from the same launches
+    # barriers; CUDA events on the grid's stream, on staged steps around every
+    # launch, so that the whole run and the kernel's own durations come from the
+    # same launches
     g.step(args.warmup)
     g.sync()
     torch.cuda.synchronize()
     barrier(dist)
     torch.cuda.synchronize()
     with ClockSampler(local) as clk:
-        kt, ms = g.step_timed(args.steps, with_total=True)
+        ms, kt = timed_steps(g, args.steps)
         torch.cuda.synchronize()
     barrier(dist)
     g.sync()
     ms_max = max_over_ranks(dist, ms, dev)
     value = aggregate(w.ncells, args.steps, ms_max, ws)
-    ab, roof = roofline_of(w, g, kt, planes=tuning["best"] if tuning and tuning["best"] else 24,
-                           item_planes=tuning["item_planes"] if tuning else (args.item_planes or 8))
+    ab, roof, launches = roofline_of_run(w, g, args.steps, ms, kt, tuning, args.item_planes or 8)
     state_bytes = (9 + 3) * 4 * ab["points"]
-    launches = sum(v[1] for v in kt.values())
     g.close()
     del g
     torch.cuda.empty_cache()
@@ -633,10 +674,8 @@ def run_batch_overhead(args):
 
 
 def run_config(w, steps, warmup=5, two_step=True, autotune_steps=0):
-    """GPU throughput of tf_step on one workload, timed whole with CUDA events
-    on the handle's stream; beside it the staged kernels' own launches
-    (tf_step_timed, which grids that tf_step runs in place take as well): their
-    algorithmic bytes over the mean launch time give the roofline object."""
+    """GPU throughput of tf_step on one workload, timed with CUDA events on the
+    handle's stream, and the roofline object of the kernels that ran."""
     import torch
     from paper_2305_13419_gb300 import twofluid as tf
     g = tf.Grid.from_workload(w)
@@ -649,12 +688,9 @@ def run_config(w, steps, warmup=5, two_step=True, autotune_steps=0):
     g.step(warmup)
     g.sync()
     torch.cuda.synchronize()
-    ms = g.time_steps(steps)
+    ms, kt = timed_steps(g, steps)
     g.sync()
-    kt, _ = g.step_timed(max(20, steps // 10), with_total=True)
-    g.sync()
-    _, roof = roofline_of(w, g, kt, planes=tuning["best"] if tuning and tuning["best"] else 24,
-                          item_planes=tuning["item_planes"] if tuning else 8)
+    _, roof, _ = roofline_of_run(w, g, steps, ms, kt, tuning)
     g.close()
     del g
     torch.cuda.empty_cache()
