@@ -606,8 +606,8 @@ def run_batch(args, plain_gcells, plain_workload="cpw-512x256x128"):
 
 
 def run_batch_singles(args):
-    """The batch's grids stepped one at a time (each alone on the GPU, single
-    steps): the per-grid rate that the batched stepping is compared with."""
+    """The batch's grids stepped one at a time by tf_step (each alone on the
+    GPU): the per-grid rate that the batched stepping is compared with."""
     import time
     import torch
     from paper_2305_13419_gb300 import twofluid as tf
@@ -615,7 +615,7 @@ def run_batch_singles(args):
     rows, cells, secs = [], 0, 0.0
     for w in W.cpw_batch()[:args.batch_singles]:
         g = tf.Grid.from_workload(w)
-        g.set_two_step(0)   # single steps, as in the batched launch
+        g.set_two_step(0)   # no two-step passes, as in the batched run
         g.step(20)
         g.sync()
         t0 = time.perf_counter()
@@ -635,9 +635,10 @@ def run_batch_singles(args):
 
 def run_batch_overhead(args):
     """The batched kernel against the single-grid kernel on the same grid:
-    tf_batch_run of a one-grid list and tf_step (single steps), each timed
-    with CUDA events on the grid's stream, on the 512 x 256 x 128 and
-    1024 x 512 x 256 CPWs.  One JSON line."""
+    tf_batch_run of a one-grid list and tf_step (single steps), both by the
+    staged kernels (a wait limit of the grid's own keeps it from stepping in
+    place), each timed with CUDA events on the grid's stream, on the
+    512 x 256 x 128 and 1024 x 512 x 256 CPWs.  One JSON line."""
     import torch
     from paper_2305_13419_gb300 import twofluid as tf
     from paper_2305_13419_gb300 import workloads as W
@@ -645,6 +646,7 @@ def run_batch_overhead(args):
     for w in (W.cpw(), W.cpw_large()):
         g = tf.Grid.from_workload(w)
         g.set_two_step(0)
+        g.set_wait_limit(1 << 23)
         g.step(6)
         g.sync()
         st = g.stream
