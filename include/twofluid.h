@@ -245,13 +245,13 @@ tf_status tf_batch_step(const tf_handle* hs, int n, int64_t nsteps);
  * a CUDA graph and replayed (the step number lives on the device and a
  * one-thread launch advances it after each step).  Every grid ends with the
  * same bits as tf_step (single steps) would give it.
- *   hs, n      handles (distinct, n <= 32768); the run is issued on hs[0]'s
- *              stream after every handle's stream has been synchronised, and
- *              synchronises it;
+ *   hs, n      handles (distinct, n <= 32768); the run begins after every
+ *              handle's stream has been synchronised and is done on return
+ *              (the one launch per step is issued on hs[0]'s stream);
  *   scratch    caller-owned device memory (256-byte aligned) of at least
  *              tf_batch_scratch_size bytes: the per-grid arguments, the work
  *              list and the source amplitudes of every step (TF_ENOMEM if
- *              smaller).
+ *              smaller).  Grids that step in place leave it untouched.
  * Creating the CUDA graph may make the CUDA runtime allocate. */
 tf_status tf_batch_scratch_size(const tf_handle* hs, int n, int64_t nsteps, size_t* bytes);
 tf_status tf_batch_run(const tf_handle* hs, int n, int64_t nsteps, void* scratch, size_t bytes);
@@ -297,10 +297,11 @@ tf_status tf_checkpoint_load(tf_handle h, const void* src, size_t bytes, int on_
  *   The handle must hold the state at rest before its first step (level 0,
  *   not yet stepped; fields as set, normally zero) with materials, sources
  *   and probes configured; no Mur walls (TF_ENOTSUP).  The call runs nsteps
- *   forward, saving a checkpoint every `segment` steps into the scratch,
- *   then walks the segments backwards: each is recomputed from its
- *   checkpoint with E kept at every level, and the transposed step runs back
- *   through it, summing per-edge gradients in FP64.  The recompute of the
+ *   forward in segments of `segment` steps, then walks them backwards: the
+ *   transposed step runs back through each, from E at every level of it, and
+ *   sums per-edge gradients in FP64.  The forward run keeps E of the last two
+ *   segments and a checkpoint (in the scratch) at the start of each one
+ *   before them, from which that one is recomputed.  The recompute of the
  *   segment before runs on a second stream of the library's (created and
  *   destroyed by the call) beside those transposed steps, into the other of
  *   two history buffers.  The adjoint's seed is
@@ -331,8 +332,8 @@ tf_status tf_fit_q(tf_handle h, int id, double f_guess, double q_guess, double* 
  * check of the step loop): sum of squares, largest magnitude and number of
  * NaN / Inf values of component comp over all storage points, in SI units.
  * E is read at the current integer level, B and Js at the half level the
- * state holds them (n - 1/2).  Uses a scratch area of the workspace (one
- * partial per z plane).  Synchronises the stream; any output may be NULL. */
+ * state holds them (n - 1/2).  Uses a scratch area of the workspace (partials
+ * of parts of the z planes).  Synchronises the stream; any output may be NULL. */
 tf_status tf_field_stats(tf_handle h, int comp, double* sumsq, double* maxabs, int64_t* nonfinite);
 
 /* Allocation-free twin of tf_field_stats.  The paper has no counterpart: it

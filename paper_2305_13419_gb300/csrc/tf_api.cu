@@ -1914,8 +1914,8 @@ tf_status tf_adjoint_run(tf_handle h, int64_t nsteps, int probe, int freq_index,
     // keeping E at every level) runs on a second stream, beside the adjoint
     // steps of segment s on the handle's stream: the two touch different
     // memory (the grid's fields / the adjoint state; each its own history
-    // buffer).  The recompute's step kernel takes one CTA per SM, leaving
-    // the rest of each SM to the adjoint passes.
+    // buffer).  Steps in place share the SMs with the adjoint passes as their
+    // CTAs come; the staged step kernel takes one CTA per SM.
     AdjStreams X;
     if (first_kept > 0 && !X.create()) return TF_ECUDA;   // (two segments at most: nothing to recompute)
     cudaStream_t const user = h->stream;

@@ -321,9 +321,10 @@ def batch_step(grids, nsteps: int):
 
 
 def batch_run(grids, nsteps: int):
-    """Advance every grid of `grids` by nsteps with one launch per step over
-    all of them (tf_batch_run): one work list over all grids' items, the
-    steps replayed from a CUDA graph.  Synchronises."""
+    """Advance every grid of `grids` by nsteps (tf_batch_run): grid by grid in
+    place, on a few streams of the library's, or (grids too large for that, or
+    a wait limit of a grid's own) with one launch per step over all of them.
+    Synchronises."""
     import torch
     hs = (C.c_void_p * len(grids))(*[g.h for g in grids])
     n = C.c_size_t()
@@ -462,9 +463,11 @@ class Grid:
         return e0.elapsed_time(e1)
 
     def step_timed(self, nsteps: int, with_total: bool = False):
-        """Advance like step(); returns {kernel: (mean ms per launch, launches)}
-        for the single-step kernel ("step") and the two-step kernel ("step2")
-        (and, with_total, also the whole run's event time in ms)."""
+        """Advance to the bits of step() by the staged kernels, which step() does
+        not take on grids that it runs in place (time_steps times those);
+        returns {kernel: (mean ms per launch, launches)} for the single-step
+        kernel ("step") and the two-step kernel ("step2") (and, with_total, also
+        the whole run's event time in ms)."""
         ms = (C.c_double * 3)()
         cnt = (C.c_int64 * 3)()
         tot = C.c_double()
@@ -474,9 +477,10 @@ class Grid:
         return (kt, tot.value) if with_total else kt
 
     def set_two_step(self, planes):
-        """Two-step passes (temporal blocking): False / 0 forbids them, True
-        allows them with 24-plane work items (the default), 4 .. 24 sets the
-        work-item length."""
+        """Two-step passes (temporal blocking): False / 0 forbids them; True asks
+        for them with 24-plane work items, 4 .. 24 with items of that length, also
+        on grids that step faster in place.  By default tf_step takes them only
+        where they are the faster ones."""
         if planes is True:
             planes = 24
         _check(load().tf_set_two_step(self.h, int(planes or 0)), "tf_set_two_step")
