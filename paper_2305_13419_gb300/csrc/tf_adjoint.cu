@@ -213,18 +213,18 @@ __device__ __forceinline__ void edge(const AdjArgs& A, const Quad& u, int e, con
         g[0] = g0;
         g[1] = g1;
     }
-    Q4 en1 = mul4(ca, ep);
+    Q4 sum = d;   // Eh = ca Eh' + (cj Jh + d): one rounding of Eh's size
     const Q4 cjm = sel4(cj, z, m);
     if (any4(cjm)) {   // a superconducting edge
         const Q4 jo = ldo(S.J[e], o), jh = sub4(jo, ev);
         sto(S.J[e], o, sel4(jh, jo, m));
-        en1 = fma4(cj, jh, en1);
+        sum = fma4(cj, jh, d);
         double* const g = S.gK[e] + o / 4u;
 #pragma unroll
         for (int p = 0; p < 4; ++p)
             if ((m >> p & 1u) && lane(cj, p) > 0.f) g[p] = fma(widen(lane(jh, p)), widen(lane(en, p)), g[p]);
     }
-    en1 = add4(en1, d);
+    Q4 en1 = fma4(ca, ep, sum);
     if (e == A.probe_comp && A.probe_o - o < 16u) {   // the objective's derivative at the probe
         const int p = (int)(A.probe_o - o) >> 2;
         const float v = p == 0 ? lane(en1, 0) : p == 1 ? lane(en1, 1) : p == 2 ? lane(en1, 2) : lane(en1, 3);
@@ -318,8 +318,8 @@ __device__ __forceinline__ void edges(const AdjArgs& A, const Quad& u) {
 }  // namespace
 
 // Face pass: Bh'tot and psi_Bh'tot.  Edge pass: Jh, psi_Eh, Eh, e; per-edge
-// gradients; the objective's derivative at the probe.  Bound by memory: 40
-// bytes a point for the faces; 72 for the edges (Bh, Eh, E^n, E^{n+1}, e) and 48
+// gradients; the objective's derivative at the probe.  Bound by memory: 36
+// bytes a point for the faces (e; Bh read and written); 72 for the edges (Bh, Eh, E^n, E^{n+1}, e) and 48
 // for the FP64 sums, with the per-point coefficients where the material
 // varies.  On the 256 x 128 x 64 CPW an adjoint step (both passes; no
 // recompute) takes 85 us; it took 125 with twelve stored weight arrays and
