@@ -380,7 +380,7 @@ __device__ __forceinline__ void sample(const PassArgs& A, int t, int k0, int k1)
 // of its one round of loads on small grids (two launches, 7.5 us a step on the
 // 128 x 64 x 40 CPW) and by memory on large ones: over the whole 512 x 256 x 128
 // CPW it takes 234 us a step (6.2 TB/s of 72 bytes per point plus the CPML
-// memories), 199 in windows of planes (below: L2 to SM traffic and the
+// memories), 189 in windows of planes (below: L2 to SM traffic and the
 // launches' ends), on the 256 x 128 x 64 CPW, whose 90 MB nearly stay in L2, 31.  What is spilled goes to
 // L2 and back: with all three slab axes' memories and Js fetched up front the E
 // pass spilled 170 bytes a thread (252 and 43 us); now the first slab axis is
@@ -453,7 +453,8 @@ cudaError_t launch_pass_probes(const Probes& R, const float* samples, long long 
 // B of that plane and the one below, and neither is a level ahead.  Every value
 // is the one of whole passes, whatever the windows.  (A periodic z axis would
 // need the last plane's neighbour before its own step.)
-// us per step of CPW grids, whole / in windows of some million points, 16 steps:
+// us per step of CPW grids, whole / in windows of some million points, 16 steps,
+// items of 2 to 4 planes:
 //   512 x 256 x 128   234 / 1.5: 208, 2: 199, 2.5: 205, 3: 220, 4: 242
 //   256 x 256 x 128   127 / 1: 120, 1.5: 105, 2: 102, 2.5: 105, 3: 118
 //   700 x 300 x 150   (421 in two-step passes) / 1.5: 387, 1.9: 368, 2.5: 372, 3: 398
