@@ -158,10 +158,10 @@ tf_status tf_add_probe(tf_handle h, int comp, const int p[3], const double* freq
  * update with CPML memory, the Js update, the theta-scheme E update with
  * sources, the Mur walls, the probe DFTs and the non-finite watchdog.  Grids
  * of up to some 80 million points run in place, a B pass and an E pass per
- * step, but for large ones that two-step passes (tf_set_two_step) step faster;
- * larger ones take those or one fused launch per step.  The results are the
- * same bits.  Asynchronous; launch errors are
- * returned (the handle is then unusable), device-side errors latch for
+ * step, but for calls on large ones that two-step passes (tf_set_two_step)
+ * step faster; larger ones take those or one fused launch per step.  The
+ * results are the same bits.  Asynchronous; launch errors are returned (the
+ * handle is then unusable), device-side errors latch for
  * tf_sync(). */
 tf_status tf_step(tf_handle h, int64_t nsteps);
 

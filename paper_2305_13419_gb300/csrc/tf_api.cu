@@ -884,16 +884,21 @@ cudaError_t run_narrow(tf_ctx* h, const Sources& S, int64_t nsteps) {
 // random material 650 / 831.  Windows of planes beyond some 0.45 M points lose a
 // little as well, with CPML: 1024 x 512 x 150 831 / 810, 720 x 720 x 110 610 / 591,
 // but 1024 x 512 x 100 568 / 577, with walls 1024 x 512 x 150 685 / 718 (smaller
-// planes: 640 x 640 x 190 809 / 818, 900 x 400 x 200 CPW 906 / 969).
-bool two_step_pays(const tf_ctx* h) {
+// planes: 640 x 640 x 190 809 / 818, 900 x 400 x 200 CPW 906 / 969).  Windows of m
+// steps cost some 1 / 4 m more than windows of many: calls of 2 steps 700 x 700 x
+// 80 495 / 462, 640 x 640 x 190 925 / 818, of 4 some 860 / 818, but of 3, where
+// two-step passes end in a single step, 881 / 883.  nsteps: the steps of the call.
+bool two_step_pays(const tf_ctx* h, int64_t nsteps) {
     const Params& P = h->P;
-    if (!h->two_step_on || !h->box_ok || !P.uniform_mu || P.per[0]) return false;
+    if (!h->two_step_on || !h->box_ok || !P.uniform_mu || P.per[0] || nsteps < 2) return false;
     const double cells = (double)h->L.ncell, plane = (double)P.n[0] * P.n[1];
     const double box = (double)(h->tx1 - h->tx0) * kSX * (h->ty1 - h->ty0) * kSY * (h->tz1 - h->tz0);
     if (box < 0.5 * cells) return false;
     const double sxy = 2.0 * P.L[0] / P.n[0] + 2.0 * P.L[1] / P.n[1], sz = 2.0 * P.L[2] / P.n[2];
     const double gain = 1e-6 * cells * (2.6 - 10.0 * sxy - 4.0 * sz - 6.0 * h->varying);
-    return h->L.pwin == h->L.kend ? gain > 50.0 : plane > 4.5e5 && sxy > 0.0 && gain > 100.0;
+    if (h->L.pwin == h->L.kend) return gain > 50.0;
+    if (nsteps < 8 && nsteps % 2 == 0) return gain > (nsteps == 2 ? 20.0 : 90.0);
+    return plane > 4.5e5 && sxy > 0.0 && gain > 100.0;
 }
 
 // May steps in place take the grid (tf_pass.cu)?  Not under a wait limit of the
@@ -901,13 +906,13 @@ bool two_step_pays(const tf_ctx* h) {
 // place / in two-step passes on a CPW grid of 134 M cells 1620 / 1512.
 bool may_pass(const tf_ctx* h) { return h->P.wait_polls == kSpinLimit && h->L.total <= kPassPoints; }
 
-// Does tf_step run in place?  Not when two-step passes were asked for.  us per step
+// Does tf_step run a call of nsteps in place?  Not when two-step passes were asked for.  us per step
 // in place / single staged steps / two-step passes on CPW grids: 0.3 M cells 7.5 /
 // 21 / 68, 2.1 M 31 / 72 / 126, 4 M 56 / 104 / 149, 8 M 101 / 165 / 182, 17 M 189 /
 // 266 / 272, 32 M 364 / - / 448, 72 M 906 / - / 969.
-bool in_place(const tf_ctx* h) {
+bool in_place(const tf_ctx* h, int64_t nsteps) {
     const bool asked = h->two_step_on == 2 && h->box_ok && h->P.uniform_mu;
-    return !asked && may_pass(h) && !two_step_pays(h);
+    return !asked && may_pass(h) && !two_step_pays(h, nsteps);
 }
 
 bool two_step(const tf_ctx* h) { return h->two_step_on && h->box_ok && h->P.uniform_mu && h->nitems_t > 0; }
@@ -1070,7 +1075,7 @@ tf_status tf_step(tf_handle h, int64_t nsteps) {
     }
     Sources S;
     fill_sources(h, S);
-    if (in_place(h)) {
+    if (in_place(h, nsteps)) {
         TF_CUDA(narrow(h) ? run_narrow(h, S, nsteps) : run_passes(h, S, nsteps));
         return TF_OK;
     }
@@ -1115,7 +1120,7 @@ tf_status tf_two_step_box(tf_handle h, int lo[3], int hi[3], int* active) {
     hi[1] = h->ty1 * kSY;
     lo[2] = h->tz0;
     hi[2] = h->tz1;
-    if (active) *active = two_step(h) && !in_place(h) ? 1 : 0;
+    if (active) *active = two_step(h) && !in_place(h, INT64_MAX - 1) ? 1 : 0;   // (in a long call)
     return TF_OK;
 }
 

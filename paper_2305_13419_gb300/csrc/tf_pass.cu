@@ -460,13 +460,14 @@ cudaError_t launch_pass_probes(const Probes& R, const float* samples, long long 
 //   700 x 300 x 150   (421 in two-step passes) / 1.5: 387, 1.9: 368, 2.5: 372, 3: 398
 //   160 x 160 x 128    53 / 1: 48, 1.4: 44, 1.8: 42;   128^3  30 / 1: 38, 1.4: 30
 // smaller windows leave the last wave of each launch emptier, larger ones leave
-// L2.  8 steps instead of 16 are 1 to 3 % slower, 4 steps 4 to 7 %.
+// L2.  8 steps instead of 16 are 1 to 3 % slower, 4 steps 4 to 7 %; one step alone
+// takes the grid whole (512 x 256 x 128 CPW 268 us in windows, 640 x 640 x 190 1044).
 // Items of one plane: with items of 2 or 4 planes a window of 5 leaves a fifth to
 // two fifths of the threads idle (1024 x 400 x 180: 756 us a step against 900).
 constexpr int kWindowSteps = 16;
 // steps of a window, of `steps` in all: groups of one size
-int window_steps(const PassArgs& A, int steps) {
-    if (A.win == A.kend) return 1;
+int window_steps(int win, const PassArgs& A, int steps) {
+    if (win == A.kend) return 1;
     const int groups = (steps + kWindowSteps - 1) / kWindowSteps;
     return (steps + groups - 1) / groups;
 }
@@ -486,14 +487,14 @@ cudaError_t launch_passes(const PassArgs& A, const Probes& R, const PassAmps* am
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     const bool early = A.nbx * A.nby * A.nbz <= kEarlyMin * A.sms;
-    const int depth = window_steps(A, steps);
+    const int win = steps > 1 ? A.win : A.kend, depth = window_steps(win, A, steps);
     cfg.numAttrs = 0;   // the first launch waits for whatever the stream holds
     cudaError_t e = cudaSuccess;
     for (int t0 = 0; t0 < steps; t0 += depth) {
         const int m = steps - t0 < depth ? steps - t0 : depth;
-        for (int z = 0; z < A.kend + m - 1; z += A.win)
+        for (int z = 0; z < A.kend + m - 1; z += win)
             for (int u = 0; u < m && e == cudaSuccess; ++u) {
-                const int k0 = z > u ? z - u : 0, k1 = z + A.win - u < A.kend ? z + A.win - u : A.kend;
+                const int k0 = z > u ? z - u : 0, k1 = z + win - u < A.kend ? z + win - u : A.kend;
                 if (k0 >= k1) continue;
                 const PassAmps& W = amp[t0 + u];
                 cfg.gridDim.z = ((k1 - k0 - 1) >> A.sc) + 1;

@@ -26,6 +26,33 @@ def test_flat_grids_give_the_bits_of_staged_steps(case):
     _same(g, ref, w, 41)
 
 
+def _uniform(n, bc, varying, default):
+    from paper_2305_13419_gb300 import twofluid as tf
+    from paper_2305_13419_gb300 import workloads as W
+    d = (10e-9, 12e-9, 8e-9)
+    cpml = tuple(W.default_cpml(6, d[a], 1e12) if bc[a] == C else None for a in range(3))
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    g = tf.Grid(n, d, 1.0, bc, cpml, courant=0.9)
+    cells = (n[2], n[1], n[0])
+    eps = torch.full(cells, 2.5, device="cuda")
+    if varying:
+        eps += torch.rand(cells, generator=gen, device="cuda")
+    g.set_materials(eps, torch.ones_like(eps), torch.zeros_like(eps), torch.zeros_like(eps))
+    if not default:
+        g.set_two_step(False)
+    for c in range(6):
+        g.set_field(c, (torch.rand(g.shape, generator=gen, device="cuda") - 0.5) * W.FIELD_SCALE[c])
+    return g
+
+
+def _same_on_device(g, h):
+    a, b = (torch.empty(x.shape, device="cuda") for x in (g, h))
+    for c in range(6):
+        g.field(c, out=a)
+        h.field(c, out=b)
+        assert torch.equal(a, b), c
+
+
 @pytest.mark.parametrize("n,bc,varying,two", [((512, 512, 128), (C, C, P), False, True), ((512, 512, 128), (C, C, P), True, False),
                                               ((256, 512, 128), (C, C, P), False, False), ((512, 512, 128), (P, C, P), False, False),
                                               ((800, 800, 80), (W_, W_, W_), False, True), ((512, 512, 128), (C, C, C), False, False),
@@ -33,29 +60,22 @@ def test_flat_grids_give_the_bits_of_staged_steps(case):
 def test_where_two_step_passes_pay(n, bc, varying, two):
     """tf_step's choice between steps in place and two-step passes where
     neither was asked for, and the same bits either way."""
-    from paper_2305_13419_gb300 import twofluid as tf
-    from paper_2305_13419_gb300 import workloads as W
-    d = (10e-9, 12e-9, 8e-9)
-    cpml = tuple(W.default_cpml(6, d[a], 1e12) if bc[a] == C else None for a in range(3))
-    grids = []
-    for default in (True, False):
-        gen = torch.Generator(device="cuda").manual_seed(5)
-        g = tf.Grid(n, d, 1.0, bc, cpml, courant=0.9)
-        cells = (n[2], n[1], n[0])
-        eps = torch.full(cells, 2.5, device="cuda")
-        if varying:
-            eps += torch.rand(cells, generator=gen, device="cuda")
-        g.set_materials(eps, torch.ones_like(eps), torch.zeros_like(eps), torch.zeros_like(eps))
-        if not default:
-            g.set_two_step(False)
-        for c in range(6):
-            g.set_field(c, (torch.rand(g.shape, generator=gen, device="cuda") - 0.5) * W.FIELD_SCALE[c])
+    grids = [_uniform(n, bc, varying, default) for default in (True, False)]
+    for g in grids:
         g.step(5)
         g.sync()
-        grids.append(g)
     assert [g.two_step_box()[1] for g in grids] == [two, False]
-    a, b = (torch.empty(g.shape, device="cuda") for g in grids)
-    for c in range(6):
-        grids[0].field(c, out=a)
-        grids[1].field(c, out=b)
-        assert torch.equal(a, b), c
+    _same_on_device(*grids)
+
+
+@pytest.mark.parametrize("n,bc", [((700, 700, 80), (C, C, C)), ((512, 512, 128), (C, C, P))])
+def test_short_calls_mix_the_routes(n, bc):
+    """Calls of one step (whole passes), of two (a two-step pass) and of more
+    in turn, against one call in place."""
+    g, ref = _uniform(n, bc, False, True), _uniform(n, bc, False, False)
+    for m in (1, 2, 3, 1, 4, 2):
+        g.step(m)
+    ref.step(13)
+    g.sync()
+    ref.sync()
+    _same_on_device(g, ref)
