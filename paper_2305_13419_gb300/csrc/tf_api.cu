@@ -906,13 +906,21 @@ bool two_step_pays(const tf_ctx* h, int64_t nsteps) {
 // place / in two-step passes on a CPW grid of 134 M cells 1620 / 1512.
 bool may_pass(const tf_ctx* h) { return h->P.wait_polls == kSpinLimit && h->L.total <= kPassPoints; }
 
+bool captured(cudaStream_t st) {
+    cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &c) != cudaSuccess) cudaGetLastError();
+    return c == cudaStreamCaptureStatusActive;
+}
+
 // Does tf_step run a call of nsteps in place?  Not when two-step passes were asked for.  us per step
 // in place / single staged steps / two-step passes on CPW grids: 0.3 M cells 7.5 /
 // 21 / 68, 2.1 M 31 / 72 / 126, 4 M 56 / 104 / 149, 8 M 101 / 165 / 182, 17 M 189 /
 // 266 / 272, 32 M 364 / - / 448, 72 M 906 / - / 969.
+// A call that is being captured runs in place wherever it may: the staged route
+// may have to build its work lists, which waits for the stream.
 bool in_place(const tf_ctx* h, int64_t nsteps) {
     const bool asked = h->two_step_on == 2 && h->box_ok && h->P.uniform_mu;
-    return !asked && may_pass(h) && !two_step_pays(h, nsteps);
+    return !asked && may_pass(h) && (!two_step_pays(h, nsteps) || captured(h->stream));
 }
 
 bool two_step(const tf_ctx* h) { return h->two_step_on && h->box_ok && h->P.uniform_mu && h->nitems_t > 0; }

@@ -79,3 +79,23 @@ def test_short_calls_mix_the_routes(n, bc):
     g.sync()
     ref.sync()
     _same_on_device(g, ref)
+
+
+def test_a_captured_call_runs_in_place():
+    """A call that would take two-step passes, captured on a handle that has
+    stepped in place only (no work lists yet)."""
+    st = torch.cuda.Stream()
+    with torch.cuda.stream(st):
+        g = _uniform((512, 512, 128), (C, C, P), False, True)
+        g.step(1)
+        g.sync()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=st):
+        g.step(2)
+    graph.replay()
+    torch.cuda.synchronize()
+    ref = _uniform((512, 512, 128), (C, C, P), False, False)
+    ref.step(3)
+    ref.sync()
+    assert g.level == 3
+    _same_on_device(g, ref)
