@@ -281,14 +281,14 @@ def cpu_baseline(w, budget_s=10.0):
 
 
 def large_block(nx=256, ny=256, nz=128):
-    """A cell block of the 1024 x 512 x 256 CPW cut around the in-port /
+    """A cell block of the timed CPW cut around the in-port /
     resonator gap at the film plane, closed with PEC walls: the bounded
     sample the FP64 oracle steps on the host cores."""
     from paper_2305_13419_gb300 import workloads as W
     w = headline_workload()
-    x0, y0 = 256 - nx // 2 + 128, 256 - ny // 2
+    x0, y0 = 256 - nx // 2 + 128, w.n[1] // 2 - ny // 2
     sl = (slice(0, nz), slice(y0, y0 + ny), slice(x0, x0 + nx))
-    return W.Workload(name=f"cpw-1024x512x256[{x0}:{x0 + nx},{y0}:{y0 + ny},0:{nz}]", n=(nx, ny, nz), d=w.d,
+    return W.Workload(name=f"{w.name}[{x0}:{x0 + nx},{y0}:{y0 + ny},0:{nz}]", n=(nx, ny, nz), d=w.d,
                       theta=w.theta, bc=("pec", "pec", "pec"), eps_r=np.ascontiguousarray(w.eps_r[sl]),
                       mu_r=np.ascontiguousarray(w.mu_r[sl]), lambda_L=np.ascontiguousarray(w.lambda_L[sl]),
                       sigma=np.ascontiguousarray(w.sigma[sl]), courant=w.courant)
@@ -475,7 +475,7 @@ def run_ours(args, ws, rank, local):
     base = None
     if rank == 0 and ws == 1 and not args.no_cpu_baseline:
         base = cpu_baseline(large_block(), budget_s=args.cpu_budget)
-        base["sample"] += " (a 256 x 256 x 128 block of the 1024 x 512 x 256 workload, PEC-closed)"
+        base["sample"] += " (a 256 x 256 x 128 block of the workload, PEC-closed)"
 
     adj = batch = extra = None
     w_name = w.name
